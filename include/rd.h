@@ -107,7 +107,11 @@ rd_status rd_build_transfer_loss(int m, int16_t *A_dev, int64_t lda, cudaStream_
  * C[i][j] = min_t (A[i][t] + B[t][j]), for an M x K matrix A, a K x N matrix B
  * and an M x N result C (C may not alias A or B).  Operands follow the
  * conventions above; result entries with no finite term are RD_INF (K = 0
- * gives an all-RD_INF C).  Runs on the DPX add-min units (__viaddmin_s16x2).
+ * gives an all-RD_INF C).  Large products are first tried on the tensor cores
+ * (entries below a window encoded as powers of two; exact wherever the sums that
+ * it finds stay within the window), tile by tile; the other tiles, and other
+ * products, run on the DPX add-min units (__viaddmin_s16x2).  The result is the
+ * same either way.
  * min_out, if not null, is a device int32 that receives min_ij C[i][j]
  * (RD_INF when C has no finite entry); it is written by this call.
  * M = 1 goes to rd_minplus_gemv.  Products whose 128 x 256 output tiles fill
@@ -182,10 +186,12 @@ rd_status rd_minplus_gemv(const int16_t *x, const int16_t *B, int64_t ldb, int16
 /*
  * rd_minplus_gemm_batched -- `count` (<= 128) independent products
  * C_i = A_i (x) B_i, each with the conventions of rd_minplus_gemm (min_out may
- * be null), in one persistent launch: two CTAs per SM walk the concatenated
- * tile list of all products, longest tiles (largest K) first, so small products
- * run side by side and the tail of a large one is filled by others.  The
- * problem table travels in the kernel's parameters (no device copy).
+ * be null), in one persistent launch over the tensor cores (one CTA per SM, in
+ * pairs) and one over the DPX units for the tiles that those leave (two per SM):
+ * each walks the concatenated tile list of all products, longest tiles (largest
+ * K) first, so small products run side by side and the tail of a large one is
+ * filled by others.  The problem table travels in the kernel's parameters (no
+ * device copy).
  */
 typedef struct {
   const int16_t *A;

@@ -1,7 +1,8 @@
 // minplus_gemm.cu -- C = A (x) B, C[i][j] = min_t (A[i][t] + B[t][j]) (Sec. 3),
-// on int16 operands with the DPX fused add-min __viaddmin_s16x2.
+// on int16 operands: large products on the tensor cores where the operands' values let them decide the result
+// (minplus_tc.cuh), everything else with the DPX fused add-min __viaddmin_s16x2.
 //
-// Design (sm_103a):
+// Design of the DPX tile (sm_103a):
 //  * Two output columns share one 32-bit register: acc = (C[i][j], C[i][j+1]).
 //    One DPX instruction updates both with min(a + b, acc), where b holds
 //    (B[t][j], B[t][j+1]) -- the natural packing of row-major B -- and a holds
@@ -25,10 +26,18 @@
 //    whose terms all involve RD_INF ends exactly at RD_INF.
 #include <cooperative_groups.h>
 
+#include <type_traits>
+
+#include "minplus_tc.cuh"
 #include "rd_internal.cuh"
 
 namespace rd {
 namespace {
+
+constexpr int16_t kMark = 0x7FFF;  // above every result entry
+// Which tiles a DPX launch computes: all; those whose first entry of C holds kMark, left by the tensor-core launch
+// before it; or those, with their first copies started before that launch has ended.
+constexpr int kUnmarked = 0, kMarked = 1, kMarkedEarly = 2;
 
 constexpr int BM = 128, BN = 256, BK = 32, NT = 256;
 constexpr int BSTAGES = 3;
@@ -57,15 +66,22 @@ __device__ __forceinline__ uint32_t pack2(int16_t lo, int16_t hi) {
   return (uint32_t)(uint16_t)lo | ((uint32_t)(uint16_t)hi << 16);
 }
 
+__device__ __forceinline__ bool tile_marked(const int16_t* c) { return *(volatile const int16_t*)c == kMark; }
+// Programmatic dependent launch: the launch before this one in the stream has ended and its writes are visible.
+__device__ __forceinline__ void after_previous_launch() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // One BM x BN output tile of C = A (x) B at (m0, n0), plus its contribution to the
 // minimum (min_out) and the diagonal minimum (diag_out) when those are not null.  SPLIT: the tile
 // of this CTA's K slice is left in shared memory ([BM][BN/2] packed words) for a cluster reduction.
-template <bool SPLIT = false, int BNT = BN>
-__device__ __forceinline__ void gemm_tile(const int16_t* __restrict__ Ag, const int16_t* __restrict__ Bg,
+//
+// EARLY: the tile may have been computed by an earlier launch (below); its copies are started before that launch has
+// ended, and false is returned when `mark`, its first entry of C, turns out not to be marked.
+template <bool SPLIT = false, int BNT = BN, bool EARLY = false>
+__device__ __forceinline__ bool gemm_tile(const int16_t* __restrict__ Ag, const int16_t* __restrict__ Bg,
                                           int16_t* __restrict__ Cg, const int64_t M, const int64_t N,
                                           const int64_t K, const int64_t lda, const int64_t ldb, const int64_t ldc,
                                           const int64_t m0, const int64_t n0, int32_t* min_out, int32_t* diag_out,
-                                          uint32_t* smem) {
+                                          uint32_t* smem, const int16_t* mark = nullptr) {
   constexpr int BSW = BK * (BNT / 2);  // one B stage, in words
   constexpr int NBC = BNT / 64;        // 16-byte chunks of a B stage per thread
   constexpr int CPR = BNT / 8;         // 16-byte chunks per B row
@@ -173,6 +189,13 @@ __device__ __forceinline__ void gemm_tile(const int16_t* __restrict__ Ag, const 
     store_a_smem(0);
   }
   if (KT > 1) load_a_regs(1);
+  if (EARLY) {
+    after_previous_launch();
+    if (!tile_marked(mark)) {
+      cp_async_wait<0>();
+      return false;
+    }
+  }
   cp_async_wait<BSTAGES - 2>();
   __syncthreads();
 
@@ -222,7 +245,7 @@ __device__ __forceinline__ void gemm_tile(const int16_t* __restrict__ Ag, const 
       for (int part = 0; part < PARTS; ++part)
         T[(ty * 8 + r) * (BNT / 8) + part * 16 + tx] =
             make_uint4(acc[r][part * 4], acc[r][part * 4 + 1], acc[r][part * 4 + 2], acc[r][part * 4 + 3]);
-    return;
+    return true;
   }
 
   // ---- epilogue: store, and reduce the minimum and the diagonal minimum
@@ -277,6 +300,7 @@ __device__ __forceinline__ void gemm_tile(const int16_t* __restrict__ Ag, const 
       if (want_diag && bd < kInf) atomicMin(diag_out, bd);
     }
   }
+  return true;
 }
 
 // Grouped rasterisation: consecutive tiles cover kGroupM row tiles x a run of column tiles, so a
@@ -291,7 +315,43 @@ __device__ __forceinline__ void grouped_tile(int64_t linear, int64_t gx, int64_t
   *tile_n = in_group / group_rows;
 }
 
-template <bool RING, int BNT = BN>
+// 16-byte vector c8 (columns n0 + 8 c8 ..) of row `row` of the tile at (m0, n0): stored to C, its entries inside
+// M x N folded into vmin / emin.
+__device__ __forceinline__ void store_vec(const GemmParams& p, int64_t m0, int64_t n0, int row, int c8, const uint4& r,
+                                          uint32_t& vmin, int32_t& emin) {
+  const int64_t gi = m0 + row, gj = n0 + c8 * 8;
+  if (gi >= p.M || gj >= p.N) return;
+  if (gj + 8 <= p.N) {
+    *reinterpret_cast<uint4*>(p.C + gi * p.ldc + gj) = r;
+    vmin = __vmins2(__vmins2(vmin, r.x), __vmins2(__vmins2(r.y, r.z), r.w));
+  } else {
+    const uint32_t w[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+    for (int e = 0; e < 8; ++e)
+      if (gj + e < p.N) {
+        const int32_t x = (int32_t)((w[e >> 1] >> (16 * (e & 1))) & 0xFFFF);
+        p.C[gi * p.ldc + gj + e] = (int16_t)x;
+        emin = min(emin, x);
+      }
+  }
+}
+
+// Folds a thread's minimum of the entries it wrote into min_out (one atomic per warp).
+__device__ __forceinline__ void fold_min_out(int32_t* min_out, uint32_t vmin, int32_t emin) {
+  int32_t lm = min(emin, min((int32_t)(vmin & 0xFFFF), (int32_t)(vmin >> 16)));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) lm = min(lm, __shfl_xor_sync(0xFFFFFFFFu, lm, o));
+  if ((threadIdx.x & 31) == 0 && lm < kInf) atomicMin(min_out, lm);
+}
+
+// Leaves a 128 x 256 tile to the DPX launch (whose tiles are BN or BN_NARROW columns wide).  By one thread, behind
+// the CTA's own stores to the tile.
+__device__ __forceinline__ void mark_tile(const GemmParams& p, int64_t m0, int64_t n0) {
+  if (m0 >= p.M) return;
+  for (int64_t n = n0; n < n0 + BN && n < p.N; n += BN_NARROW) p.C[m0 * p.ldc + n] = kMark;
+}
+
+template <bool RING, int BNT, int MARKED>
 __global__ void __launch_bounds__(NT, BNT == BN ? 2 : 3) minplus_gemm_kernel(GemmParams p) {
   extern __shared__ __align__(16) uint32_t smem[];
   const int16_t* Ag = p.A;
@@ -305,15 +365,19 @@ __global__ void __launch_bounds__(NT, BNT == BN ? 2 : 3) minplus_gemm_kernel(Gem
   }
   int64_t tm, tn;
   grouped_tile((int64_t)blockIdx.y * gridDim.x + blockIdx.x, gridDim.x, gridDim.y, &tm, &tn);
-  gemm_tile<false, BNT>(Ag, p.B, Cg, p.M, p.N, p.K, p.lda, p.ldb, p.ldc, tm * BM, tn * BNT, p.min_out, p.diag_out,
-                        smem);
+  if (MARKED == kMarked) {
+    after_previous_launch();
+    if (!tile_marked(p.C + tm * BM * p.ldc + tn * BNT)) return;
+  }
+  gemm_tile<false, BNT, MARKED == kMarkedEarly>(Ag, p.B, Cg, p.M, p.N, p.K, p.lda, p.ldb, p.ldc, tm * BM, tn * BNT,
+                                                p.min_out, p.diag_out, smem, p.C + tm * BM * p.ldc + tn * BNT);
 }
 
 // ---- split K for small products: a cluster of S CTAs per output tile, CTA r computing the tile over
 // its K slice [r kslice, (r + 1) kslice); the S partial tiles, left in the CTAs' shared memory, meet in
 // distributed shared memory, CTA r min-reducing rows [r BM/S, (r + 1) BM/S) of the tile and writing
 // them (with the minimum).  Used when the output tiles alone would not fill one wave of the GPU.
-template <int BNT>
+template <int BNT, int MARKED>
 __global__ void __launch_bounds__(NT, BNT == BN ? 2 : 3) minplus_gemm_splitk_kernel(GemmParams p, int64_t kslice) {
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
@@ -322,9 +386,15 @@ __global__ void __launch_bounds__(NT, BNT == BN ? 2 : 3) minplus_gemm_splitk_ker
   int64_t tm, tn;
   grouped_tile((int64_t)blockIdx.y * gridDim.x + blockIdx.x, gridDim.x, gridDim.y, &tm, &tn);
   const int64_t m0 = tm * BM, n0 = tn * BNT;
+  // an unmarked tile ends the whole cluster (every CTA of it reads the mark before C is written, after its barrier)
+  if (MARKED == kMarked) {
+    after_previous_launch();
+    if (!tile_marked(p.C + m0 * p.ldc + n0)) return;
+  }
   const int64_t k0 = (int64_t)rank * kslice, k1 = (k0 + kslice < p.K) ? k0 + kslice : p.K;
-  gemm_tile<true, BNT>(p.A + k0, p.B + k0 * p.ldb, nullptr, p.M, p.N, k1 - k0, p.lda, p.ldb, p.ldc, m0, n0, nullptr,
-                       nullptr, smem);
+  if (!gemm_tile<true, BNT, MARKED == kMarkedEarly>(p.A + k0, p.B + k0 * p.ldb, nullptr, p.M, p.N, k1 - k0, p.lda,
+                                                    p.ldb, p.ldc, m0, n0, nullptr, nullptr, smem, p.C + m0 * p.ldc + n0))
+    return;
   cluster.sync();  // every partial tile is in place
   const int rows = BM / S;
   uint32_t vmin = kInf2;
@@ -370,6 +440,73 @@ __global__ void __launch_bounds__(NT, BNT == BN ? 2 : 3) minplus_gemm_splitk_ker
   cluster.sync();  // no CTA leaves while others may still read its shared memory
 }
 
+// ---- the tensor cores first (minplus_tc.cuh).  A 128 x 256 part that they do not decide is marked in C, and the DPX
+// launch that follows computes the marked parts only.
+static_assert(BM == tc::kBM && BN == tc::kBN, "the DPX tile is the part that is marked");
+
+// What a CTA does with its half of a pair's tile, by the producers: writes the decided parts to C, computes their few
+// undecided outputs term by term (a warp each), marks the others.
+template <int NH>
+__device__ __forceinline__ void tc_finish(const GemmParams& p, bool ok, int64_t m0, int64_t n0, const char* buf,
+                                          const tc::Shared* s) {
+  uint32_t vmin = kInf2;
+  int32_t emin = kInf;
+  const uint4* T = reinterpret_cast<const uint4*>(buf);
+  bool skip[NH];
+#pragma unroll
+  for (int h = 0; h < NH; ++h) skip[h] = !ok || s->cnt[h] > (uint32_t)tc::kMostFix;
+  for (int v = threadIdx.x; v < BM * 32 * NH; v += tc::kProducers) {
+    const int row = v / (32 * NH), c8 = v % (32 * NH);
+    if (!skip[NH == 1 ? 0 : c8 >> 5]) store_vec(p, m0, n0, row, c8, T[row * (32 * NH) + (c8 ^ (row & 7))], vmin, emin);
+  }
+#pragma unroll
+  for (int h = 0; h < NH; ++h) {
+    if (skip[h]) {
+      if (threadIdx.x == 0) mark_tile(p, m0, n0 + h * BN);
+    } else if (s->cnt[h] > 0) {
+      tc::producers_sync();  // the undecided outputs' placeholders are written
+      for (uint32_t i = threadIdx.x >> 5; i < s->cnt[h]; i += tc::kProducers / 32) {
+        const int64_t gi = m0 + (s->list[h][i] >> 9), gj = n0 + (s->list[h][i] & 511u);
+        const int32_t x = tc::dot(p.A + gi * p.lda, p.B + gj, p.ldb, p.K);
+        if ((threadIdx.x & 31) == 0) p.C[gi * p.ldc + gj] = (int16_t)x;
+        emin = min(emin, x);
+      }
+    }
+  }
+  if (p.min_out != nullptr) fold_min_out(p.min_out, vmin, emin);
+  tc::producers_sync();  // the tile and its counts are read: the next tile may overwrite them
+}
+
+// The buffer of the stages inside the kernel's shared memory (1024-byte aligned).
+__device__ __forceinline__ char* tc_buffer(char* smem) {
+  return smem + ((1024u - (smem_u32(smem) & 1023u)) & 1023u);
+}
+
+// Pair c takes tiles c, c + pairs, ... of the gx x gy tiles of 256 x 256 NH in the grouped order.
+template <int NH>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc::kThreads, 1)
+    minplus_tc_kernel(GemmParams p, tc::Code code, int64_t gx, int64_t gy) {
+  extern __shared__ __align__(16) char tc_smem[];
+  __shared__ tc::Shared ts;
+  const int64_t rank = tc::cta_rank(), pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
+  if (!tc::worth(p, code.W, &ts)) {
+    for (int64_t t = pair + threadIdx.x * pairs; t < gx * gy; t += tc::kThreads * pairs)
+      for (int h = 0; h < NH; ++h) mark_tile(p, (t / gx * 2 + rank) * BM, (t % gx * NH + h) * BN);
+    return;
+  }
+  char* buf = tc_buffer(tc_smem);
+  tc::open<NH>(&ts);
+  tc::Progress pr;
+  for (int64_t t = pair; t < gx * gy; t += pairs) {
+    int64_t tm, tn;
+    grouped_tile(t, gx, gy, &tm, &tn);
+    const int64_t m0 = (tm * 2 + rank) * BM, n0 = tn * NH * BN;
+    const bool ok = tc::tile<NH>(p, m0, n0, code, buf, &ts, pr);
+    if (threadIdx.x < tc::kProducers) tc_finish<NH>(p, ok, m0, n0, buf, &ts);
+  }
+  tc::close<NH>(&ts);
+}
+
 // ---- stream-K for products with few output tiles.  The units of work are (output tile, k-tile) pairs,
 // tile by tile in the grouped order; a grid of exactly the resident CTAs (two per SM) takes equal
 // contiguous runs of them, so every SM does the same number of add-mins whatever the tile count.  A run
@@ -399,25 +536,10 @@ __device__ __forceinline__ uint32_t sk_first_unit(uint32_t c, uint32_t U, uint32
 __device__ __forceinline__ uint32_t sk_cta_of(uint32_t u, uint32_t U, uint32_t G) { return ((u + 1) * G - 1) / U; }
 
 // Writes vector v of a 128 x 256 tile at (m0, n0) of C (the layout gemm_tile<true> leaves in shared
-// memory: row v / 32, columns (v % 32 / 16) * 128 + (v % 16) * 8 ..), folding its entries into vmin/emin.
+// memory: row v / 32, columns 8 (v % 32) ..).
 __device__ __forceinline__ void sk_store(const GemmParams& p, int64_t m0, int64_t n0, int v, const uint4& r,
                                          uint32_t& vmin, int32_t& emin) {
-  const int row = v / (BN / 8), c8 = v % (BN / 8);
-  const int64_t gi = m0 + row, gj = n0 + (c8 / 16) * 128 + (c8 % 16) * 8;
-  if (gi >= p.M || gj >= p.N) return;
-  if (gj + 8 <= p.N) {
-    *reinterpret_cast<uint4*>(p.C + gi * p.ldc + gj) = r;
-    vmin = __vmins2(__vmins2(vmin, r.x), __vmins2(__vmins2(r.y, r.z), r.w));
-  } else {
-    const uint32_t w[4] = {r.x, r.y, r.z, r.w};
-#pragma unroll
-    for (int e = 0; e < 8; ++e)
-      if (gj + e < p.N) {
-        const int32_t x = (int32_t)((w[e >> 1] >> (16 * (e & 1))) & 0xFFFF);
-        p.C[gi * p.ldc + gj + e] = (int16_t)x;
-        emin = min(emin, x);
-      }
-  }
+  store_vec(p, m0, n0, v / (BN / 8), v % (BN / 8), r, vmin, emin);
 }
 
 // The segment a CTA works on: its first unit and the tile's coordinates, derived from the CTA's run.
@@ -437,14 +559,6 @@ __device__ __forceinline__ SkSeg sk_segment(const StreamK& sk, uint32_t u, uint3
   g.m0 = (int64_t)(first_m + in_group % group_rows) * BM;
   g.n0 = (int64_t)(in_group / group_rows) * BN;
   return g;
-}
-
-// Folds a thread's minimum of the entries it wrote into min_out (one atomic per warp).
-__device__ __forceinline__ void sk_min_out(int32_t* min_out, uint32_t vmin, int32_t emin) {
-  int32_t lm = min(emin, min((int32_t)(vmin & 0xFFFF), (int32_t)(vmin >> 16)));
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) lm = min(lm, __shfl_xor_sync(0xFFFFFFFFu, lm, o));
-  if ((threadIdx.x & 31) == 0 && lm < kInf) atomicMin(min_out, lm);
 }
 
 __global__ void __launch_bounds__(NT, 2) minplus_gemm_streamk_kernel(GemmParams p, StreamK sk) {
@@ -507,7 +621,7 @@ __global__ void __launch_bounds__(NT, 2) minplus_gemm_streamk_kernel(GemmParams 
         if (threadIdx.x == 0) sk.cnt[g.t] = 0u;  // every contributor has arrived: ready for the next launch
       }
     }
-    if (p.min_out != nullptr) sk_min_out(p.min_out, vmin, emin);
+    if (p.min_out != nullptr) fold_min_out(p.min_out, vmin, emin);
     __syncthreads();  // the partial tile is read before the next segment's prologue overwrites it
     if (threadIdx.x == 0) s_u = uu + (g.kb - g.ka);
     __syncthreads();
@@ -525,32 +639,97 @@ struct BatchProblem {
   int64_t lda, ldb, ldc, M, N, K;
   int32_t* min_out;
   int64_t tiles_m, tiles_n;
+  tc::Code code;  // L = 0: DPX only
 };
 
 struct BatchParams {
   int count;
   int64_t tile_start[kMaxBatch + 1];  // prefix sums of the tile counts, in schedule order
+  int64_t tc_start[kMaxBatch + 1];    // of the tensor-core tile counts (none for DPX-only products)
   BatchProblem p[kMaxBatch];
 };
+
+__device__ __forceinline__ int batch_problem_of(const BatchParams& bp, int64_t t) {
+  int lo = 0, hi = bp.count - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (bp.tile_start[mid] <= t) lo = mid;
+    else hi = mid - 1;
+  }
+  return lo;
+}
 
 // CTA c takes tiles c, c + gridDim.x, ... of the concatenated tile list.  Problems are
 // ordered by decreasing K (tile cost), so the round robin hands out the long tiles first.
 __global__ void __launch_bounds__(NT, 2) minplus_gemm_batched_kernel(const __grid_constant__ BatchParams bp) {
   extern __shared__ __align__(16) uint32_t smem[];
   const int64_t total = bp.tile_start[bp.count];
+  after_previous_launch();
   for (int64_t t = blockIdx.x; t < total; t += gridDim.x) {
-    int lo = 0, hi = bp.count - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (bp.tile_start[mid] <= t) lo = mid;
-      else hi = mid - 1;
-    }
+    const int lo = batch_problem_of(bp, t);
     const BatchProblem& q = bp.p[lo];
     int64_t tm, tn;
     grouped_tile(t - bp.tile_start[lo], q.tiles_n, q.tiles_m, &tm, &tn);
+    if (q.code.L && !tile_marked(q.C + tm * BM * q.ldc + tn * BN)) continue;
     __syncthreads();  // the previous tile's shared memory is no longer read
     gemm_tile(q.A, q.B, q.C, q.M, q.N, q.K, q.lda, q.ldb, q.ldc, tm * BM, tn * BN, q.min_out, nullptr, smem);
   }
+}
+
+// The same schedule on the tensor cores, before it: pairs, and tiles of 256 x 256 NH.
+template <int NH>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc::kThreads, 1)
+    minplus_tc_batched_kernel(const __grid_constant__ BatchParams bp) {
+  extern __shared__ __align__(16) char tc_smem[];
+  __shared__ tc::Shared ts;
+  // the current product and tile: kept out of the registers
+  __shared__ GemmParams p;
+  __shared__ tc::Code code;
+  __shared__ int cur, changed, worth;
+  __shared__ int64_t at[2];
+  char* buf = tc_buffer(tc_smem);
+  if (threadIdx.x == 0) cur = -1;
+  tc::open<NH>(&ts);
+  tc::Progress pr;
+#pragma unroll 1
+  for (int64_t t = blockIdx.x >> 1; t < bp.tc_start[bp.count]; t += gridDim.x >> 1) {
+    __syncthreads();  // everybody is done with the previous tile
+    if (threadIdx.x == 0) {
+      int i = cur < 0 ? 0 : cur;
+      while (bp.tc_start[i + 1] <= t) ++i;
+      const BatchProblem& q = bp.p[i];
+      changed = i != cur;
+      cur = i;
+      int64_t tm, tn;
+      grouped_tile(t - bp.tc_start[i], (q.N + NH * BN - 1) / (NH * BN), (q.M + 2 * BM - 1) / (2 * BM), &tm, &tn);
+      at[0] = (tm * 2 + tc::cta_rank()) * BM;
+      at[1] = tn * NH * BN;
+      code = q.code;
+      p.A = q.A;
+      p.lda = q.lda;
+      p.B = q.B;
+      p.ldb = q.ldb;
+      p.C = q.C;
+      p.ldc = q.ldc;
+      p.M = q.M;
+      p.N = q.N;
+      p.K = q.K;
+      p.min_out = q.min_out;
+    }
+    __syncthreads();
+    if (changed) {
+      const bool w = tc::worth(p, code.W, &ts);
+      if (threadIdx.x == 0) worth = w;
+      __syncthreads();
+    }
+    if (worth) {
+      const bool ok = tc::tile<NH>(p, at[0], at[1], code, buf, &ts, pr);
+      if (threadIdx.x < tc::kProducers) tc_finish<NH>(p, ok, at[0], at[1], buf, &ts);
+    } else if (threadIdx.x < NH) {
+      mark_tile(p, at[0], at[1] + threadIdx.x * BN);
+    }
+  }
+  tc::close<NH>(&ts);
 }
 
 struct MinOutList {
@@ -665,34 +844,59 @@ __global__ void __launch_bounds__(kGemvThreads) minplus_gemv_kernel(const int16_
   }
 }
 
-template <int WHICH>  // 0 plain, 1 ring, 2 batched, 3 split K, 4 plain narrow, 5 split K narrow, 6 stream-K
-cudaError_t set_smem_attr() {
+// Raises a kernel's dynamic shared memory limit, once per kernel and device.
+template <auto KERNEL>
+cudaError_t set_smem_attr(size_t bytes) {
   static int done_dev[64] = {0};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev >= 0 && dev < 64 && done_dev[dev]) return cudaSuccess;
-  if (WHICH == 0)
-    e = cudaFuncSetAttribute(minplus_gemm_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
-  else if (WHICH == 1)
-    e = cudaFuncSetAttribute(minplus_gemm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
-  else if (WHICH == 3)
-    e = cudaFuncSetAttribute(minplus_gemm_splitk_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)SMEM_BYTES);
-  else if (WHICH == 4)
-    e = cudaFuncSetAttribute(minplus_gemm_kernel<false, BN_NARROW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem_bytes(BN_NARROW));
-  else if (WHICH == 5)
-    e = cudaFuncSetAttribute(minplus_gemm_splitk_kernel<BN_NARROW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem_bytes(BN_NARROW));
-  else if (WHICH == 6)
-    e = cudaFuncSetAttribute(minplus_gemm_streamk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)SMEM_BYTES);
-  else
-    e = cudaFuncSetAttribute(minplus_gemm_batched_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)SMEM_BYTES);
+  e = cudaFuncSetAttribute(KERNEL, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   if (e == cudaSuccess && dev >= 0 && dev < 64) done_dev[dev] = 1;
   return e;
+}
+
+// Launches KERNEL with its shared memory limit raised; S > 1: clusters of S CTAs along z.
+// after_tc: the launch for the marked tiles, which may start before the tensor-core launch has ended.
+template <auto KERNEL, class... Args>
+cudaError_t launch_kernel(dim3 grid, int threads, size_t smem, int S, bool after_tc, cudaStream_t s,
+                          const Args&... args) {
+  cudaError_t e = set_smem_attr<KERNEL>(smem);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[2];
+  cfg.attrs = attr;
+  if (S > 1) {
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 1;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = (unsigned)S;
+    cfg.numAttrs = 1;
+  }
+  if (after_tc) {
+    attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[cfg.numAttrs].val.programmaticStreamSerializationAllowed = 1;
+    ++cfg.numAttrs;
+  }
+  e = cudaLaunchKernelEx(&cfg, KERNEL, args...);
+  return e == cudaSuccess ? cudaGetLastError() : e;
+}
+
+int sm_count() {
+  int dev = 0, sms = 148;
+  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return sms;
+}
+
+// The encoding of a product; L = 0 where the tensor-core tile does not apply.
+tc::Code tc_code(int64_t K, int64_t lda, int64_t ldb) {
+  if (K < tc::kMinK || K > tc::kMaxK || lda > tc::kMaxLd || ldb > tc::kMaxLd) return tc::Code{0, 0};
+  return tc::code_for(K);
 }
 
 }  // namespace
@@ -706,9 +910,7 @@ cudaError_t launch_fill_i32(int32_t* dst, int32_t value, cudaStream_t s) {
 // smallest that fills it, with every K slice at least 8 k-tiles deep and none empty.  (Shorter slices
 // measured slower: at N = 1024, 8 slices of 128 took 0.051 ms against 0.045 ms for 4 of 256.)
 int splitk_factor(int64_t tiles, int64_t K) {
-  int dev = 0, sms = 148;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int64_t wave = 2 * (int64_t)sms;
+  const int64_t wave = 2 * (int64_t)sm_count();
   int S = 1;
   while (S < 8 && tiles * S < wave && K >= (int64_t)(2 * S) * 8 * BK) S *= 2;
   if (S > 1) {
@@ -727,7 +929,8 @@ bool splitk_suits(int S, int64_t K) {
 
 int64_t gemm_tiles(int64_t M, int64_t N) { return ((M + BM - 1) / BM) * ((N + BN - 1) / BN); }
 
-cudaError_t launch_minplus_gemm(const GemmParams& p, bool ring, cudaStream_t s, int force_splitk, int force_tile) {
+cudaError_t launch_minplus_gemm(const GemmParams& p, bool ring, cudaStream_t s, int force_splitk, int force_tile,
+                                bool marked) {
   int S = 1;     // ring mode and the diagonal output keep one CTA per tile (no diagonal in the split form)
   int tile = 0;  // 0: BM x BN, 1: BM x BN_NARROW (no ring mode, no diagonal)
   if (force_splitk > 0) {
@@ -750,43 +953,51 @@ cudaError_t launch_minplus_gemm(const GemmParams& p, bool ring, cudaStream_t s, 
   const int64_t gx = (p.N + bn - 1) / bn, gy = (p.M + BM - 1) / BM;
   if (gx <= 0 || gy <= 0) return cudaSuccess;
   if (gx > 0x7FFFFFFF || gy > 65535) return cudaErrorInvalidConfiguration;
-  const dim3 grid((unsigned)gx, (unsigned)gy);
-  cudaError_t e;
-  if (S > 1) {
-    e = tile ? set_smem_attr<5>() : set_smem_attr<3>();
+  const dim3 grid((unsigned)gx, (unsigned)gy, (unsigned)S);
+  const int64_t kslice = ((p.K + S - 1) / S + BK - 1) / BK * BK;
+  auto launch = [&](auto bnt, auto marked) {
+    constexpr int kBnt = decltype(bnt)::value, kMode = decltype(marked)::value;
+    return S > 1 ? launch_kernel<minplus_gemm_splitk_kernel<kBnt, kMode>>(grid, NT, smem, S, kMode != kUnmarked, s, p, kslice)
+                 : launch_kernel<minplus_gemm_kernel<false, kBnt, kMode>>(grid, NT, smem, 1, kMode != kUnmarked, s, p);
+  };
+  auto with_tile = [&](auto marked) {
+    return tile ? launch(std::integral_constant<int, BN_NARROW>{}, marked) : launch(std::integral_constant<int, BN>{}, marked);
+  };
+  if (ring) return launch_kernel<minplus_gemm_kernel<true, BN, kUnmarked>>(grid, NT, smem, 1, false, s, p);
+  if (!marked) return with_tile(std::integral_constant<int, kUnmarked>{});
+  // few waves: the copies of a CTA's first stages cost less than the wait for the mark that they hide
+  return gx * gy * S <= 8 * (int64_t)sm_count() ? with_tile(std::integral_constant<int, kMarkedEarly>{})
+                                                : with_tile(std::integral_constant<int, kMarked>{});
+}
+
+// Where operands with large entries make the look at a sample pointless, it costs 4 to 8 us, 3 % of the DPX product at
+// N = 2048 and 0.3 % at 4096 (2195 us); where the tensor cores do the work, 288 us become 35 and 2195 become 129.
+constexpr double kTcMinWork = 8589934592.0;  // 2048^3
+
+// The tensor-core launch of a product (not in ring mode, no diagonal), and the DPX launch for what it left.
+cudaError_t launch_minplus_product(const GemmParams& p, cudaStream_t s) {
+  bool marked = false;
+  const tc::Code code = tc_code(p.K, p.lda, p.ldb);
+  if (code.L && (double)p.M * (double)p.N * (double)p.K > kTcMinWork) {
+    const int64_t pairs = sm_count() / 2, gy = (p.M + 2 * BM - 1) / (2 * BM), KT = (p.K + tc::kBK - 1) / tc::kBK;
+    // the width with the shorter schedule: rounds of the pairs x clocks of one tile
+    int nh = 1;
+    int64_t best = 0, gx = 0;
+    for (int h = 1; h <= 2; ++h) {
+      const int64_t x = (p.N + h * BN - 1) / (h * BN);
+      const int64_t cost = (x * gy + pairs - 1) / pairs * (h == 1 ? 900 * KT + 5000 : 1450 * KT + 9000);
+      if (h == 1 || cost < best) best = cost, nh = h, gx = x;
+    }
+    const int64_t n = gx * gy < pairs ? gx * gy : pairs;
+    const cudaError_t e =
+        nh == 1 ? launch_kernel<minplus_tc_kernel<1>>(dim3((unsigned)(2 * n)), tc::kThreads, tc::smem_bytes(1), 1, false, s, p,
+                                                      code, gx, gy)
+                : launch_kernel<minplus_tc_kernel<2>>(dim3((unsigned)(2 * n)), tc::kThreads, tc::smem_bytes(2), 1, false, s, p,
+                                                      code, gx, gy);
     if (e != cudaSuccess) return e;
-    const int64_t kslice = ((p.K + S - 1) / S + BK - 1) / BK * BK;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)gx, (unsigned)gy, (unsigned)S);
-    cfg.blockDim = dim3(NT, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 1;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = (unsigned)S;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    e = tile ? cudaLaunchKernelEx(&cfg, minplus_gemm_splitk_kernel<BN_NARROW>, p, kslice)
-             : cudaLaunchKernelEx(&cfg, minplus_gemm_splitk_kernel<BN>, p, kslice);
-    if (e != cudaSuccess) return e;
-    return cudaGetLastError();
+    marked = true;
   }
-  if (ring) {
-    e = set_smem_attr<1>();
-    if (e != cudaSuccess) return e;
-    minplus_gemm_kernel<true><<<grid, NT, SMEM_BYTES, s>>>(p);
-  } else if (tile) {
-    e = set_smem_attr<4>();
-    if (e != cudaSuccess) return e;
-    minplus_gemm_kernel<false, BN_NARROW><<<grid, NT, smem, s>>>(p);
-  } else {
-    e = set_smem_attr<0>();
-    if (e != cudaSuccess) return e;
-    minplus_gemm_kernel<false><<<grid, NT, SMEM_BYTES, s>>>(p);
-  }
-  return cudaGetLastError();
+  return launch_minplus_gemm(p, false, s, 0, 0, marked);
 }
 
 }  // namespace rd
@@ -814,7 +1025,7 @@ extern "C" rd_status rd_minplus_gemm(const int16_t* A, int64_t lda, const int16_
   GemmParams p{};
   p.A = A; p.lda = lda; p.B = B; p.ldb = ldb; p.C = C; p.ldc = ldc;
   p.M = M; p.N = N; p.K = K; p.min_out = min_out; p.diag_out = nullptr;
-  e = launch_minplus_gemm(p, false, s);
+  e = launch_minplus_product(p, s);
   if (e != cudaSuccess) { set_cuda_error(e); return RD_ERR_CUDA; }
   return RD_OK;
 }
@@ -892,11 +1103,7 @@ extern "C" rd_status rd_minplus_gemm_streamk(const int16_t* A, int64_t lda, cons
   sk.U = (uint32_t)units;
   sk.part = static_cast<uint4*>(work);
   sk.cnt = reinterpret_cast<uint32_t*>(static_cast<char*>(work) + L.part_bytes);
-  e = set_smem_attr<6>();
-  if (e == cudaSuccess) {
-    minplus_gemm_streamk_kernel<<<(unsigned)L.grid, NT, SMEM_BYTES, s>>>(p, sk);
-    e = cudaGetLastError();
-  }
+  e = launch_kernel<minplus_gemm_streamk_kernel>(dim3((unsigned)L.grid), NT, SMEM_BYTES, 1, false, s, p, sk);
   if (e != cudaSuccess) { set_cuda_error(e); return RD_ERR_CUDA; }
   return RD_OK;
 }
@@ -1096,21 +1303,24 @@ extern "C" rd_status rd_minplus_gemm_batched(const rd_gemm_problem* problems, in
     b.min_out = q.min_out;
     b.tiles_m = (q.M + BM - 1) / BM;
     b.tiles_n = (q.N + BN - 1) / BN;
+    b.code = tc_code(q.K, q.lda, q.ldb);
     bp.tile_start[bp.count + 1] = bp.tile_start[bp.count] + b.tiles_m * b.tiles_n;
+    const int64_t tcs = b.code.L ? (q.M + 2 * BM - 1) / (2 * BM) * ((q.N + 2 * BN - 1) / (2 * BN)) : 0;
+    bp.tc_start[bp.count + 1] = bp.tc_start[bp.count] + tcs;
     ++bp.count;
   }
   fill_min_outs_kernel<<<1, 128, 0, s>>>(mins);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) { set_cuda_error(e); return RD_ERR_CUDA; }
   if (bp.count == 0) return RD_OK;
-  e = set_smem_attr<2>();
-  if (e != cudaSuccess) { set_cuda_error(e); return RD_ERR_CUDA; }
-  int dev = 0, sms = 148;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int sms = sm_count();
   const int64_t total = bp.tile_start[bp.count];
   const int64_t grid = total < 2 * (int64_t)sms ? total : 2 * (int64_t)sms;  // two resident CTAs per SM
-  minplus_gemm_batched_kernel<<<(unsigned)grid, NT, SMEM_BYTES, s>>>(bp);
-  e = cudaGetLastError();
+  const int64_t tcs = bp.tc_start[bp.count], pairs = tcs < sms / 2 ? tcs : sms / 2;
+  if (pairs > 0)
+    e = launch_kernel<minplus_tc_batched_kernel<2>>(dim3((unsigned)(2 * pairs)), tc::kThreads, tc::smem_bytes(2), 1, false, s,
+                                                    bp);
+  if (e == cudaSuccess) e = launch_kernel<minplus_gemm_batched_kernel>(dim3((unsigned)grid), NT, SMEM_BYTES, 1, pairs > 0, s, bp);
   if (e != cudaSuccess) { set_cuda_error(e); return RD_ERR_CUDA; }
   return RD_OK;
 }

@@ -93,7 +93,7 @@ struct GemmParams {
 // 256, 1: 128 x 128) -- the autotuner's trials; else the tuning table's factor and tile for the product's
 // size class, else the built-in rule (the wide tile).
 cudaError_t launch_minplus_gemm(const GemmParams& p, bool ring, cudaStream_t s, int force_splitk = 0,
-                                int force_tile = 0);
+                                int force_tile = 0, bool marked = false);
 bool splitk_suits(int S, int64_t K);         // S in {1, 2, 4, 8} and every K slice non-empty
 int64_t gemm_tiles(int64_t M, int64_t N);  // output tiles (CTAs of an unsplit launch)
 
