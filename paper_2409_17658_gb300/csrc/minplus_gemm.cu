@@ -396,11 +396,12 @@ __global__ void __launch_bounds__(NT, BNT == BN ? 2 : 3) minplus_gemm_splitk_ker
                                                     p.ldb, p.ldc, m0, n0, nullptr, nullptr, smem, p.C + m0 * p.ldc + n0))
     return;
   cluster.sync();  // every partial tile is in place
-  const int rows = BM / S;
+  const int rows = (BM + S - 1) / S;
   uint32_t vmin = kInf2;
   int32_t emin = kInf;
   for (int v = threadIdx.x; v < rows * (BNT / 8); v += NT) {
     const int row = rank * rows + v / (BNT / 8), c8 = v % (BNT / 8);
+    if (row >= BM) break;
     uint4 r = make_uint4(kInf2, kInf2, kInf2, kInf2);
     for (int q = 0; q < S; ++q) {
       const uint4 t = cluster.map_shared_rank(reinterpret_cast<uint4*>(smem), q)[row * (BNT / 8) + c8];
@@ -901,30 +902,63 @@ tc::Code tc_code(int64_t K, int64_t lda, int64_t ldb) {
 
 }  // namespace
 
+// The built-in launch shape of a DPX product: the tile (0: 128 x 256, 1: 128 x 128), the number of K slices S, and the
+// modeled clocks.
+struct GemmShape {
+  int S, tile;
+  double clocks;
+};
+
 cudaError_t launch_fill_i32(int32_t* dst, int32_t value, cudaStream_t s) {
   fill_i32_kernel<<<1, 1, 0, s>>>(dst, value);
   return cudaGetLastError();
 }
 
-// Split K when the output tiles alone fill less than one wave (2 CTAs per SM): S in {2, 4, 8}, the
-// smallest that fills it, with every K slice at least 8 k-tiles deep and none empty.  (Shorter slices
-// measured slower: at N = 1024, 8 slices of 128 took 0.051 ms against 0.045 ms for 4 of 256.)
-int splitk_factor(int64_t tiles, int64_t K) {
-  const int64_t wave = 2 * (int64_t)sm_count();
-  int S = 1;
-  while (S < 8 && tiles * S < wave && K >= (int64_t)(2 * S) * 8 * BK) S *= 2;
-  if (S > 1) {
-    const int64_t kslice = ((K + S - 1) / S + BK - 1) / BK * BK;
-    while (S > 1 && (int64_t)(S - 1) * kslice >= K) S /= 2;  // every slice non-empty
+static bool slices_full(int S, int64_t K) {  // every one of S K slices is non-empty
+  const int64_t kslice = ((K + S - 1) / S + BK - 1) / BK * BK;
+  return (int64_t)(S - 1) * kslice < K;
+}
+
+// The shape with the shortest modeled schedule.  A CTA's clocks are its k-tiles at the DPX rate its SM's n CTAs reach
+// together, its prologue and epilogue, and the cluster's reduction; the launch is full waves and a rest spread over
+// the SMs.  The CTAs of a cluster share a GPC (8 of them, 19 SMs): that bounds how many clusters fit with n CTAs per
+// SM, with one SM less where S is not a power of two (measured: 64 clusters of 7 do not fit in one wave).
+// The constants fit GB300's times of 12 sizes from 97 x 130 x 161 to 6000 x 5000 x 700 to 15 %.  Against the former
+// rule (wide tile, S the smallest power of two that fills a wave, slices of 256 terms and more): 97 x 130 x 161 37 ->
+// 12 us, 512^3 45 -> 17, 300 x 400 x 3000 70 -> 43, 2507 x 3001 x 1999 614 -> 520, 4096^3 2195 -> 1950; 1024^3 stays.
+GemmShape gemm_shape(int64_t M, int64_t N, int64_t K) {
+  const int64_t sms = sm_count(), gpcs = 8;
+  GemmShape best{1, 0, 0};
+  for (int tile = 0; tile < 2; ++tile) {
+    const int64_t bn = tile ? BN_NARROW : BN, cap = tile ? 3 : 2;  // CTAs per SM
+    const int64_t tiles = ((M + BM - 1) / BM) * ((N + bn - 1) / bn);
+    for (int S = 1; S <= 8; ++S) {
+      if (!slices_full(S, K)) continue;
+      const int64_t kt = ((K + S - 1) / S + BK - 1) / BK;
+      auto fits = [&](int64_t n) -> int64_t {  // tiles that run at once with n CTAs per SM
+        return S == 1 ? sms * n : (sms / gpcs - ((S & (S - 1)) != 0)) * n / S * gpcs;
+      };
+      auto clocks = [&](int64_t n) {
+        const double eff = tile ? (n == 1 ? 0.75 : 0.88) : (n == 1 ? 0.88 : 0.93);
+        return (double)(n * kt * bn * BK) / eff + 6000 + (S > 1 ? 1200 * S : 0);
+      };
+      const int64_t wave = fits(cap), rest = tiles % (wave > 0 ? wave : 1);
+      if (wave <= 0) continue;
+      double c = (double)(tiles / wave) * clocks(cap);
+      if (rest > 0) {
+        int64_t n = 1;
+        while (n < cap && fits(n) < rest) ++n;
+        c += clocks(n);
+      }
+      if (best.clocks == 0 || c < best.clocks) best = GemmShape{S, tile, c};
+    }
   }
-  return S;
+  return best;
 }
 
 bool splitk_suits(int S, int64_t K) {
   if (S == 1) return true;
-  if (S != 2 && S != 4 && S != 8) return false;
-  const int64_t kslice = ((K + S - 1) / S + BK - 1) / BK * BK;
-  return (int64_t)(S - 1) * kslice < K;
+  return (S == 2 || S == 4 || S == 8) && slices_full(S, K);
 }
 
 int64_t gemm_tiles(int64_t M, int64_t N) { return ((M + BM - 1) / BM) * ((N + BN - 1) / BN); }
@@ -945,7 +979,9 @@ cudaError_t launch_minplus_gemm(const GemmParams& p, bool ring, cudaStream_t s, 
       S = t.p[0];
       tile = t.p[1];
     } else {
-      S = splitk_factor(gemm_tiles(p.M, p.N), p.K);
+      const GemmShape g = gemm_shape(p.M, p.N, p.K);
+      S = g.S;
+      tile = g.tile;
     }
   }
   const int bn = tile ? BN_NARROW : BN;
@@ -970,32 +1006,34 @@ cudaError_t launch_minplus_gemm(const GemmParams& p, bool ring, cudaStream_t s, 
                                                 : with_tile(std::integral_constant<int, kMarked>{});
 }
 
-// Where operands with large entries make the look at a sample pointless, it costs 4 to 8 us, 3 % of the DPX product at
-// N = 2048 and 0.3 % at 4096 (2195 us); where the tensor cores do the work, 288 us become 35 and 2195 become 129.
-constexpr double kTcMinWork = 8589934592.0;  // 2048^3
-
 // The tensor-core launch of a product (not in ring mode, no diagonal), and the DPX launch for what it left.
+// Only a product whose modeled DPX schedule is kTcGain times the tensor cores' is tried: where the operands' values are
+// against it the look at a sample costs 4 us.  At the line (1.5 to 2): 700^3, 23 against 25 us, is left out; 1024^3, 25
+// against 43 (47 where the sample says no), is tried.  2048^3 takes 35 against 271, 4096^3 129 against 1946.
+constexpr double kTcGain = 1.8;
 cudaError_t launch_minplus_product(const GemmParams& p, cudaStream_t s) {
   bool marked = false;
   const tc::Code code = tc_code(p.K, p.lda, p.ldb);
-  if (code.L && (double)p.M * (double)p.N * (double)p.K > kTcMinWork) {
+  if (code.L) {
     const int64_t pairs = sm_count() / 2, gy = (p.M + 2 * BM - 1) / (2 * BM), KT = (p.K + tc::kBK - 1) / tc::kBK;
     // the width with the shorter schedule: rounds of the pairs x clocks of one tile
     int nh = 1;
     int64_t best = 0, gx = 0;
     for (int h = 1; h <= 2; ++h) {
       const int64_t x = (p.N + h * BN - 1) / (h * BN);
-      const int64_t cost = (x * gy + pairs - 1) / pairs * (h == 1 ? 900 * KT + 5000 : 1450 * KT + 9000);
+      const int64_t cost = (x * gy + pairs - 1) / pairs * (h == 1 ? 1080 * KT + 9000 : 1540 * KT + 14000);
       if (h == 1 || cost < best) best = cost, nh = h, gx = x;
     }
-    const int64_t n = gx * gy < pairs ? gx * gy : pairs;
-    const cudaError_t e =
-        nh == 1 ? launch_kernel<minplus_tc_kernel<1>>(dim3((unsigned)(2 * n)), tc::kThreads, tc::smem_bytes(1), 1, false, s, p,
-                                                      code, gx, gy)
-                : launch_kernel<minplus_tc_kernel<2>>(dim3((unsigned)(2 * n)), tc::kThreads, tc::smem_bytes(2), 1, false, s, p,
-                                                      code, gx, gy);
-    if (e != cudaSuccess) return e;
-    marked = true;
+    if (gemm_shape(p.M, p.N, p.K).clocks > kTcGain * (double)(best + 16000)) {
+      const int64_t n = gx * gy < pairs ? gx * gy : pairs;
+      const cudaError_t e =
+          nh == 1 ? launch_kernel<minplus_tc_kernel<1>>(dim3((unsigned)(2 * n)), tc::kThreads, tc::smem_bytes(1), 1,
+                                                        false, s, p, code, gx, gy)
+                  : launch_kernel<minplus_tc_kernel<2>>(dim3((unsigned)(2 * n)), tc::kThreads, tc::smem_bytes(2), 1,
+                                                        false, s, p, code, gx, gy);
+      if (e != cudaSuccess) return e;
+      marked = true;
+    }
   }
   return launch_minplus_gemm(p, false, s, 0, 0, marked);
 }

@@ -108,3 +108,20 @@ def test_entries_outside_the_range_keep_their_result(rd):
     with np.errstate(over="ignore"):
         s = np.minimum(INF, np.array([(a[i][:, None] + b).min(0) for i in range(M)], dtype=np.int16)).astype(np.int32)
     assert np.array_equal(C.cpu().numpy()[:, :N].astype(np.int32), s)
+
+
+@pytest.mark.parametrize("dist", ["u32", "wide"])
+@pytest.mark.parametrize("K", [33, 64, 65, 100, 129, 161, 193, 225, 257])
+def test_small_products_split_k_in_any_number_of_slices(rd, orc, K, dist):
+    """Few output tiles: K is cut into 2 .. 8 slices of whole k-tiles, not only powers of two, and the slices' rows of
+    the tile into uneven shares."""
+    import torch
+
+    for i, (M, N) in enumerate([(2, 8), (97, 130), (128, 128), (129, 257), (300, 201)]):
+        a, b = operands(dist, M, N, K, 40 + i)
+        C = torch.full((M, (N + 7) // 8 * 8), -7, dtype=torch.int16, device="cuda")
+        low = torch.zeros(1, dtype=torch.int32, device="cuda")
+        rd.minplus_gemm(upload(a, -3), upload(b, -5), C, M, N, K, min_out=low)
+        w, got = orc.minplus_i16(a, b), C.cpu().numpy()
+        assert np.array_equal(got[:, :N].astype(np.int32), w), (M, N, K)
+        assert (got[:, N:] == -7).all() and int(low) == int(w.min()), (M, N, K)
