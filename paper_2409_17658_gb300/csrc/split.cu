@@ -37,6 +37,7 @@
 // loop reads nothing but shared memory.  When they do not fit (very unbalanced splits), the kernel
 // reads them from global memory instead.
 #include <initializer_list>
+#include <algorithm>
 #include <mutex>
 
 #include "power_dev.cuh"
@@ -55,7 +56,6 @@ constexpr int kTauCount = 5;
 // acd}.  A group's record holds the starts of its 7 sub-lists and their end.
 constexpr int kSets = 7;
 constexpr int kRec = 8;
-constexpr int kDefaultSlabsPerCta = 8;
 __host__ __device__ constexpr int set_index(uint32_t mask) {
   return mask == 0x1 ? 0 : mask == 0x4 ? 1 : mask == 0x5 ? 2 : mask == 0x6 ? 3 : mask == 0x7 ? 4 : mask == 0xC ? 5
        : mask == 0xD ? 6 : -1;
@@ -951,6 +951,22 @@ size_t pass_smem(int max_slots, int n_groups, int max_list, int W, bool words, b
   return *staged ? full : (size_t)(max_slots + 1) * (size_t)W * 2;
 }
 
+// Slabs per CTA.  More of them spread a CTA's staging of its fiber's metadata, fewer make more CTAs and a shorter last
+// wave: the most (up to 8) that leave 2.3 full waves of CTAs (5 and 4 per SM in the two passes), in pass 2, which
+// stages less, 12 as far as 2 slabs; up to 32 where even that leaves 12.  Measured per product, against 8 always:
+// m = 6 27.9 -> 15.9 us, m = 7 82 -> 29, m = 8 168 -> 139, m = 9 1.11 -> 1.09 ms, m = 10 10.30 -> 10.18 ms.
+int default_slabs(int64_t fibers, int64_t cols, int W, bool first) {
+  int dev = 0, sms = 148;
+  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int64_t slabs = (cols + W - 1) / W, wave = (int64_t)sms * (first ? 5 : 4);
+  auto ctas = [&](int k) { return fibers * ((slabs + k - 1) / k); };
+  int k = 8;
+  while (!first && k > 2 && ctas(k) < 12 * wave) k /= 2;
+  while (k > 1 && 10 * ctas(k) < 23 * wave) k /= 2;
+  while (k >= 8 && k < 32 && ctas(2 * k) >= 12 * wave) k *= 2;
+  return k;
+}
+
 // Slab width: the widest of 256, 128, 64 columns whose staged fiber leaves room for 3 CTAs per SM (narrower
 // slabs put more groups in a warp and cost shared-memory bank conflicts; at 256 a warp folds one group at a
 // time, so its lanes never diverge: m = 8 0.186 -> 0.144 ms and m = 9 1.147 -> 1.109 ms tuned), else the
@@ -1043,6 +1059,10 @@ template <bool RING>
 cudaError_t run_passes(SplitPass p1, SplitPass p2, const rd_split_info_t& info, cudaStream_t s) {
   const int64_t N = info.N;
   const int64_t cw = info.chunk_cols > 0 ? info.chunk_cols : N;
+  if (cw < N) {  // a chunk has fewer slabs than the plan's choice was made for
+    p1.slabs_per_cta = std::min(p1.slabs_per_cta, default_slabs(info.n_sigma, cw, info.w1, true));
+    p2.slabs_per_cta = std::min(p2.slabs_per_cta, default_slabs(info.n_pi, cw, info.w2, false));
+  }
   cudaError_t e = cudaSuccess;
   for (int64_t c0 = 0; c0 < N && e == cudaSuccess; c0 += cw) {
     const int64_t w = (N - c0 < cw) ? (N - c0) : cw;
@@ -1372,8 +1392,8 @@ extern "C" rd_status rd_split_plan(int m, int j, void* plan_dev, size_t plan_byt
   info->slots2 = slots2;
   info->lmax1 = lm[0];
   info->lmax2 = lm[1];
-  info->k1 = kDefaultSlabsPerCta;
-  info->k2 = kDefaultSlabsPerCta;
+  info->k1 = default_slabs(info->n_sigma, L.N, w1, true);
+  info->k2 = default_slabs(info->n_pi, L.N, w2, false);
   info->chunk_cols = 0;
   rd_tune_entry_t t;  // a tuned launch shape for this (m, j), when its widths fit this plan
   if (tune_find(RD_TUNE_SPLIT, m, j, &t) && valid_w(t.p[0], slots1) && valid_w(t.p[2], slots2)) {
