@@ -128,8 +128,10 @@ void free_job(rd_server* sv, Job* j) {
 }
 
 // Large jobs (C_m >= kSplitN) step with the row-split product; smaller ones with the sparse one,
-// all of whose products share one launch.
-constexpr int64_t kSplitN = 4096;
+// all of whose products share one launch.  A cold batch over m = 2..8 takes 13.6 ms with m = 8 alone on the row split,
+// 12.4 with m = 7 (2507 words) too, 12.9 with m = 6 and 13.6 with all: a job's own launches then cost more than its
+// share of the common one.
+constexpr int64_t kSplitN = 2048;
 
 // The row-split operands of a large job: its plan and intermediate, after A and the work buffer.
 rd_status admit_split(rd_server* sv, Job* j, size_t base) {
