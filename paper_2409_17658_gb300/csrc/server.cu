@@ -64,6 +64,7 @@ struct Job {
   void* plan = nullptr;       // row-split plan (large jobs)
   int16_t* X = nullptr;       // its intermediate
   rd::SplitRing split{};
+  bool sparse = false;        // the row split's operands exceed the whole budget: the sparse step instead
   size_t work_bytes = 0, footprint = 0, need = 0;
   rd::RunDesc run{};
   double cost = 1.0;  // bytes one product moves: B rows (sparse: entries x N x 2; row split: 4 (N + X rows) N)
@@ -132,6 +133,9 @@ void free_job(rd_server* sv, Job* j) {
 // 12.4 with m = 7 (2507 words) too, 12.9 with m = 6 and 13.6 with all: a job's own launches then cost more than its
 // share of the common one.
 constexpr int64_t kSplitN = 2048;
+// Below this many words a job whose row-split operands (17 MB more than the sparse ones at m = 7) exceed the whole
+// budget takes the sparse step.
+constexpr int64_t kSplitOnly = 4096;
 
 // The row-split operands of a large job: its plan and intermediate, after A and the work buffer.
 rd_status admit_split(rd_server* sv, Job* j, size_t base) {
@@ -172,7 +176,7 @@ rd_status admit(rd_server* sv, Job* j) {
   rd_padded_dim(j->N, &j->ld);
   const size_t a_bytes = (size_t)j->N * (size_t)j->ld * 2;
   rd_power_work_bytes(j->N, j->ld, sv->kmax, sv->slots, &j->work_bytes);
-  const bool use_split = j->N >= kSplitN && rd_split_default_j(j->m) > 0;
+  const bool use_split = j->N >= kSplitN && !j->sparse && rd_split_default_j(j->m) > 0;
   const int64_t nb = (j->N + sv->R - 1) / sv->R;
   const size_t start_bytes = use_split ? 0 : (size_t)(nb + 1) * 8;
   const size_t base = a_bytes + j->work_bytes + start_bytes;
@@ -188,7 +192,12 @@ rd_status admit(rd_server* sv, Job* j) {
   if (rc == RD_OK) rc = rd_build_transfer(j->m, j->A, j->ld, sv->stream);
   if (use_split && rc == RD_OK) {
     rc = admit_split(sv, j, base);
-    if (rc == RD_ERR_NOMEM || rc == RD_ERR_ARG) return rc;  // freed already
+    if (rc == RD_ERR_ARG && j->N < kSplitOnly) {  // freed already
+      j->sparse = true;
+      j->need = 0;
+      return admit(sv, j);
+    }
+    if (rc == RD_ERR_NOMEM || rc == RD_ERR_ARG) return rc;
   }
   int64_t entries = 0;
   if (!use_split && rc == RD_OK) rc = rd_sparse_count(j->A, j->ld, j->N, j->N, sv->R, j->start, &entries, sv->stream);
