@@ -3,13 +3,14 @@
 Prints ONE JSON line (rank 0).  Headline: add-min throughput of the (min,+)
 product C = A (x) B at N = 16384 (synthetic operands, int16, entries uniform in
 [0, 32], each infinite with probability 1/2, seeds 1 and 2), with inputs resident
-in HBM; the step is one rd_minplus_gemm call (DPX product + fused minimum
-reduction).  Operands (2 x 512 MiB) exceed the 129 MB L2, so no flush is needed
+in HBM; the step is one rd_minplus_gemm call (the product on the tensor cores,
+the DPX launch for the tiles that they leave, the fused minimum reduction).  Operands (2 x 512 MiB) exceed the 129 MB L2, so no flush is needed
 between steps.  Beside it, in the same line:
   * e2e: the same product through the C ABI with host operands, the pinned
     host->device copies of A and B and the device->host copy of C inside the
     timed region;
-  * roofline of the product kernel against the DPX add-min peak;
+  * roofline of the product kernel against the bf16 tensor peak (one multiply-add
+    per add-min), with the DPX add-min peak beside it;
   * time_to_period: the whole hot path (enumerate + build A(G), power until the
     first repeat, gamma_R closed form) for m = 3, 7, 9, with the oracle's time;
   * cpu_baseline: the oracle's product on a bounded sample of rows.
@@ -35,13 +36,13 @@ sys.path.insert(0, ROOT)
 N_HEAD = 16384
 SEED_A, SEED_B = 1, 2
 # Nominal DPX rate from unit counts and clock: 152 SMs x 64 __viaddmin_s16x2 lanes per clock x 2 add-mins per
-# lane x 2070 MHz.  The roofline's peak is the measured one (rd_measure_addmin_peak, run by this script before
-# the timed region); the nominal figure is printed beside it.
+# lane x 2070 MHz.  frac_of_peak is against the measured one (rd_measure_addmin_peak, run by this script before
+# the timed region), which the tensor-core product exceeds; the nominal figure is printed beside it.
 SMS, DPX_LANES_PER_CLK, ADDMIN_PER_LANE, SM_MAX_MHZ = 152, 64, 2, 2070.0
 PEAK_GOPS = SMS * DPX_LANES_PER_CLK * ADDMIN_PER_LANE * SM_MAX_MHZ * 1e6 / 1e9
 # DRAM bytes (read + write) per launch of the product kernel at N = 16384, from a one-pass ncu capture of
-# dram__bytes_read.sum and dram__bytes_write.sum on that launch (8.60 GB read + 0.552 GB written).
-GEMM_TRAFFIC_BYTES = 9.152e9
+# dram__bytes_read.sum and dram__bytes_write.sum on that launch (7.54 GB read + 0.536 GB written).
+GEMM_TRAFFIC_BYTES = 8.076e9
 CONFIG_NAME = "synthetic dense (min,+) GEMM N=16384, int16 uniform[0,32], P(inf)=0.5"
 
 
@@ -56,6 +57,15 @@ def _measured_hbm_gbs() -> float:
 
 
 HBM_GBS = _measured_hbm_gbs()
+
+
+def _measured_bf16_tflops() -> float:
+    """The measured cuBLAS bf16 rate of the GB300s (MEASURED_PEAKS.json), else 1900 TFLOP/s."""
+    try:
+        with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as fh:
+            return float(json.load(fh)["bf16_tflops"])
+    except (OSError, ValueError, KeyError):
+        return 1900.0
 
 
 def max_over_ranks(value_ms: float, dist, device) -> float:
@@ -565,7 +575,7 @@ def batched_products(rd, torch, count: int = 64, seed: int = 4) -> dict:
         e1.record(stream)
         torch.cuda.synchronize()
         ms = e0.elapsed_time(e1) / reps
-        out[name] = {"ms": ms, "gops": ops / (ms * 1e-3) / 1e9, "launches": count if name.startswith("one") else 2}
+        out[name] = {"ms": ms, "gops": ops / (ms * 1e-3) / 1e9, "launches": 2 * count if name.startswith("one") else 3}
     out["speedup"] = out["one_launch_per_product"]["ms"] / out["batched_persistent"]["ms"]
     out["results_identical"] = bool(all(torch.equal(p[2][:, :p[4]], r[:, :p[4]]) for p, r in zip(probs, refs)))
     del probs, refs
@@ -1025,19 +1035,20 @@ def main() -> None:
         achieved = ops_per_step / (per_launch_ms * 1e-3) / 1e9
         per_clk = peak["addmin_per_clk_per_sm"]
         peak_max = per_clk * peak["sm_count"] * SM_MAX_MHZ * 1e6 / 1e9  # measured rate per clock at the max clock
-        roof = {"bound": "alu", "achieved": achieved, "peak": peak_max, "unit": "G add-min/s",
-                "frac": achieved / peak_max, "traffic": GEMM_TRAFFIC_BYTES,
-                "kernel": "minplus_gemm_kernel<false>", "per_launch_ms": per_launch_ms,
+        tensor_peak = _measured_bf16_tflops() * 1e3 / 2  # G multiply-adds per second: one per add-min
+        roof = {"bound": "tensor", "achieved": achieved, "peak": tensor_peak, "unit": "G add-min/s",
+                "frac": achieved / tensor_peak, "traffic": GEMM_TRAFFIC_BYTES,
+                "kernel": "minplus_tc_kernel<2>", "per_launch_ms": per_launch_ms,
                 "peak_basis": "measured",
-                "peak_how": (f"rd_measure_addmin_peak: {per_clk:.2f} add-min/clk/SM (clock64 spans of a full wave "
-                             f"of __viaddmin_s16x2 chains) x {peak['sm_count']} SMs x {SM_MAX_MHZ:.0f} MHz"),
-                "peak_measured_run": {"addmin_per_clk_per_sm": per_clk, "gops_at_run_clock": peak["addmin_per_s"] / 1e9,
-                                      "run_sm_mhz": peak["sm_mhz"], "ms": peak["ms"], "clocks": peak["clocks"]},
-                "peak_nominal": PEAK_GOPS,
-                "peak_nominal_formula": "152 SMs x 64 DPX s16x2 lanes/clk x 2 add-min x 2070 MHz",
-                "frac_of_nominal": achieved / PEAK_GOPS}
-        if clk.get("sm_mhz"):
-            roof["frac_at_sampled_clock"] = achieved / (per_clk * peak["sm_count"] * clk["sm_mhz"] * 1e6 / 1e9)
+                "peak_how": "bf16 TFLOP/s of a plain cuBLAS GEMM / 2: the kernel does one bf16 multiply-add per add-min",
+                "dpx_peak": peak_max, "frac_of_dpx_peak": achieved / peak_max,
+                "dpx_peak_how": (f"rd_measure_addmin_peak: {per_clk:.2f} add-min/clk/SM (clock64 spans of a full wave "
+                                 f"of __viaddmin_s16x2 chains) x {peak['sm_count']} SMs x {SM_MAX_MHZ:.0f} MHz"),
+                "dpx_peak_measured_run": {"addmin_per_clk_per_sm": per_clk,
+                                          "gops_at_run_clock": peak["addmin_per_s"] / 1e9,
+                                          "run_sm_mhz": peak["sm_mhz"], "ms": peak["ms"], "clocks": peak["clocks"]},
+                "dpx_peak_nominal": PEAK_GOPS,
+                "dpx_peak_nominal_formula": "152 SMs x 64 DPX s16x2 lanes/clk x 2 add-min x 2070 MHz"}
         line = {"metric": "(min,+) add-min GOPS and % of GB300 DPX/INT peak at N=16384; gamma_R time-to-period vs oracle",
                 "value": value, "unit": "G add-min/s", "n_gpus": world, "steps": args.steps, "warmup": args.warmup,
                 "ms_per_step": total_ms / args.steps, "higher_is_better": True, "scaling": "weak",
@@ -1050,7 +1061,7 @@ def main() -> None:
                         "how": "one rd_minplus_gemm_host call per step (pinned host A, B in; C out); steps "
                                "alternate two streams and staging buffers, so copies overlap the neighbouring "
                                "step's product"},
-                "gpu_launches": 2 * args.steps,
+                "gpu_launches": 3 * args.steps,  # min_out fill, tensor cores, DPX for marked tiles
                 "roofline": roof, "clocks": clk}
         line.update(extra)
         print(json.dumps(line))

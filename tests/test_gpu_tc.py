@@ -125,3 +125,25 @@ def test_small_products_split_k_in_any_number_of_slices(rd, orc, K, dist):
         w, got = orc.minplus_i16(a, b), C.cpu().numpy()
         assert np.array_equal(got[:, :N].astype(np.int32), w), (M, N, K)
         assert (got[:, N:] == -7).all() and int(low) == int(w.min()), (M, N, K)
+
+
+@pytest.mark.parametrize("kind", ["u32", "wide", "halves"])
+def test_captured_product_replays(rd, kind):
+    """Both launches of a product in a CUDA graph, replayed over a result of other values."""
+    import torch
+
+    M, N, K = 1500, 1300, 1200
+    a, b = operands(kind, M, N, K, 9)
+    A, B = upload(a, INF), upload(b, INF)
+    want, C = (torch.full((M, 1304), -7, dtype=torch.int16, device="cuda") for _ in range(2))
+    low = torch.zeros(1, dtype=torch.int32, device="cuda")
+    rd.minplus_gemm(A, B, want, M, N, K)
+    torch.cuda.synchronize()
+    stream, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        rd.minplus_gemm(A, B, C, M, N, K, min_out=low, stream=stream)
+    for _ in range(3):
+        C.fill_(0)
+        C[:, N:] = -7
+        graph.replay()
+    assert torch.equal(C, want) and int(low) == int(want[:, :N].min())
