@@ -547,7 +547,7 @@ rd_status rd_power_until_periodic_multi_bounded(rd_power_run *runs, int count, i
  * of the finite-difference equation of Prop. 7, in a few hundred bytes.  A
  * record exported by one process can be imported by another, which then answers
  * every n of that m on the host with no device work (the search costs about
- * 0.35 s and 87 GB of device memory at m = 10, 9 s and 225 GB at m = 11).
+ * 0.35 s and 61 GB of device memory at m = 10, 9 s and 225 GB at m = 11).
  * Records describe the transfer matrix of Sec. 4.A (rd_build_transfer), not the
  * Appendix variant.
  *   m      1..RD_MAX_M.
@@ -775,9 +775,9 @@ rd_status rd_measure_addmin_peak(void *work_dev, size_t work_bytes, int64_t trip
  * n >= 3).  The first call for a given m builds A(G) and runs the period
  * search: in one CTA (rd_power_until_periodic) when C_m <= 128 (m <= 4), else
  * by rd_power_until_periodic_split, on the current device, in device memory this
- * call allocates and frees (about 11 powers of C_m x C_m int16: 10 GB at m = 9,
- * 87 GB at m = 10; RD_ERR_NOMEM when that does not fit); the result (gamma for n < k + p, and (k, p, q)) is
- * cached per m for the life of the process, and later calls evaluate the
+ * call allocates and frees (about 7.3 powers of C_m x C_m int16: 7 GB at m = 9,
+ * 61 GB at m = 10; RD_ERR_NOMEM when that does not fit); the result (gamma for
+ * n < k + p, and (k, p, q)) is cached per m for the life of the process, and later calls evaluate the
  * solution of the finite-difference equation of Prop. 7 on the host:
  * gamma(n) = gamma(k + (n - k) mod p) + q floor((n - k) / p) for n >= k.
  * Thread-safe.  Synchronous.
