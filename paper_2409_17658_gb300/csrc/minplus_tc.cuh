@@ -349,7 +349,9 @@ __device__ __forceinline__ bool tile(const GemmParams& p, const int64_t m0, cons
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t rank = cta_rank();
   const int KT = (int)((p.K + kBK - 1) / kBK);
-  const int check = KT >= 16 ? KT >> 3 : -1;
+  // The early look (an eighth of the way) costs 2 us a tile, 8 % of a product at K = 1024; a tile of fewer stages than
+  // this that turns out hopeless costs at most 20.
+  const int check = KT >= 40 ? KT >> 3 : -1;
 
   if (tid == 0) s->at[0] = m0, s->at[1] = n0;
   if (tid == 0) s->bad = s->look[0] = s->look[1] = s->cnt[0] = s->cnt[1] = 0;

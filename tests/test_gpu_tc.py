@@ -2,7 +2,7 @@
 
 The batched entry point tries it for every K >= 64, so small shapes reach it.  Shapes sit at the edges of its tiles
 (256 rows and 512 columns per pair of CTAs, halves of 128 and 256), its 64-term stages and its early look (from
-16 stages on); the values decide whether an output is decided, computed term by term, or left to the DPX tile.
+40 stages on); the values decide whether an output is decided, computed term by term, or left to the DPX tile.
 """
 import numpy as np
 import pytest
@@ -11,7 +11,7 @@ pytestmark = pytest.mark.gpu
 
 INF = 0x3FFF
 SHAPES = [(1, 8, 64), (2, 9, 65), (128, 256, 64), (129, 257, 127), (256, 512, 128), (257, 513, 129), (127, 255, 192),
-          (255, 511, 191), (300, 521, 1023), (260, 515, 1024), (130, 1025, 1600)]
+          (255, 511, 191), (300, 521, 1023), (260, 515, 1024), (130, 1025, 1600), (140, 601, 2496), (257, 513, 2561)]
 
 
 @pytest.fixture(scope="module")
