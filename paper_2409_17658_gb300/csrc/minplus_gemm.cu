@@ -74,9 +74,9 @@ __device__ __forceinline__ void after_previous_launch() { asm volatile("griddepc
 // minimum (min_out) and the diagonal minimum (diag_out) when those are not null.  SPLIT: the tile
 // of this CTA's K slice is left in shared memory ([BM][BN/2] packed words) for a cluster reduction.
 //
-// EARLY: the tile may have been computed by an earlier launch (below); its copies are started before that launch has
-// ended, and false is returned when `mark`, its first entry of C, turns out not to be marked.
-template <bool SPLIT = false, int BNT = BN, bool EARLY = false>
+// MODE: the tile may have been computed by an earlier launch (below); false is returned when `mark`, its first entry
+// of C, turns out not to be marked (kMarkedEarly: its first copies are started before that launch has ended).
+template <bool SPLIT = false, int BNT = BN, int MODE = kUnmarked>
 __device__ __forceinline__ bool gemm_tile(const int16_t* __restrict__ Ag, const int16_t* __restrict__ Bg,
                                           int16_t* __restrict__ Cg, const int64_t M, const int64_t N,
                                           const int64_t K, const int64_t lda, const int64_t ldb, const int64_t ldc,
@@ -178,6 +178,11 @@ __device__ __forceinline__ bool gemm_tile(const int16_t* __restrict__ Ag, const 
 #pragma unroll
     for (int c = 0; c < NV; ++c) acc[r][c] = kInf2;
 
+  if (MODE == kMarked) {
+    after_previous_launch();
+    if (!tile_marked(mark)) return false;
+  }
+
   // ---- prologue
 #pragma unroll
   for (int s = 0; s < BSTAGES - 1; ++s) {
@@ -189,7 +194,7 @@ __device__ __forceinline__ bool gemm_tile(const int16_t* __restrict__ Ag, const 
     store_a_smem(0);
   }
   if (KT > 1) load_a_regs(1);
-  if (EARLY) {
+  if (MODE == kMarkedEarly) {
     after_previous_launch();
     if (!tile_marked(mark)) {
       cp_async_wait<0>();
@@ -365,11 +370,7 @@ __global__ void __launch_bounds__(NT, BNT == BN ? 2 : 3) minplus_gemm_kernel(Gem
   }
   int64_t tm, tn;
   grouped_tile((int64_t)blockIdx.y * gridDim.x + blockIdx.x, gridDim.x, gridDim.y, &tm, &tn);
-  if (MARKED == kMarked) {
-    after_previous_launch();
-    if (!tile_marked(p.C + tm * BM * p.ldc + tn * BNT)) return;
-  }
-  gemm_tile<false, BNT, MARKED == kMarkedEarly>(Ag, p.B, Cg, p.M, p.N, p.K, p.lda, p.ldb, p.ldc, tm * BM, tn * BNT,
+  gemm_tile<false, BNT, MARKED>(Ag, p.B, Cg, p.M, p.N, p.K, p.lda, p.ldb, p.ldc, tm * BM, tn * BNT,
                                                 p.min_out, p.diag_out, smem, p.C + tm * BM * p.ldc + tn * BNT);
 }
 
@@ -387,12 +388,8 @@ __global__ void __launch_bounds__(NT, BNT == BN ? 2 : 3) minplus_gemm_splitk_ker
   grouped_tile((int64_t)blockIdx.y * gridDim.x + blockIdx.x, gridDim.x, gridDim.y, &tm, &tn);
   const int64_t m0 = tm * BM, n0 = tn * BNT;
   // an unmarked tile ends the whole cluster (every CTA of it reads the mark before C is written, after its barrier)
-  if (MARKED == kMarked) {
-    after_previous_launch();
-    if (!tile_marked(p.C + m0 * p.ldc + n0)) return;
-  }
   const int64_t k0 = (int64_t)rank * kslice, k1 = (k0 + kslice < p.K) ? k0 + kslice : p.K;
-  if (!gemm_tile<true, BNT, MARKED == kMarkedEarly>(p.A + k0, p.B + k0 * p.ldb, nullptr, p.M, p.N, k1 - k0, p.lda,
+  if (!gemm_tile<true, BNT, MARKED>(p.A + k0, p.B + k0 * p.ldb, nullptr, p.M, p.N, k1 - k0, p.lda,
                                                     p.ldb, p.ldc, m0, n0, nullptr, nullptr, smem, p.C + m0 * p.ldc + n0))
     return;
   cluster.sync();  // every partial tile is in place
@@ -1001,8 +998,9 @@ cudaError_t launch_minplus_gemm(const GemmParams& p, bool ring, cudaStream_t s, 
   };
   if (ring) return launch_kernel<minplus_gemm_kernel<true, BN, kUnmarked>>(grid, NT, smem, 1, false, s, p);
   if (!marked) return with_tile(std::integral_constant<int, kUnmarked>{});
-  // few waves: the copies of a CTA's first stages cost less than the wait for the mark that they hide
-  return gx * gy * S <= 8 * (int64_t)sm_count() ? with_tile(std::integral_constant<int, kMarkedEarly>{})
+  // one wave: the copies of a CTA's first stages hide the wait for the mark; with 720 CTAs and none marked they
+  // cost 4 of 50 us
+  return gx * gy * S <= 2 * (int64_t)sm_count() ? with_tile(std::integral_constant<int, kMarkedEarly>{})
                                                 : with_tile(std::integral_constant<int, kMarked>{});
 }
 
