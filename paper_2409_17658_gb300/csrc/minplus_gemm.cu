@@ -899,12 +899,6 @@ tc::Code tc_code(int64_t K, int64_t lda, int64_t ldb) {
 
 }  // namespace
 
-// The built-in launch shape of a DPX product: the tile (0: 128 x 256, 1: 128 x 128), the number of K slices S, and the
-// modeled clocks.
-struct GemmShape {
-  int S, tile;
-  double clocks;
-};
 
 cudaError_t launch_fill_i32(int32_t* dst, int32_t value, cudaStream_t s) {
   fill_i32_kernel<<<1, 1, 0, s>>>(dst, value);
@@ -961,7 +955,7 @@ bool splitk_suits(int S, int64_t K) {
 int64_t gemm_tiles(int64_t M, int64_t N) { return ((M + BM - 1) / BM) * ((N + BN - 1) / BN); }
 
 cudaError_t launch_minplus_gemm(const GemmParams& p, bool ring, cudaStream_t s, int force_splitk, int force_tile,
-                                bool marked) {
+                                bool marked, const GemmShape* shape) {
   int S = 1;     // ring mode and the diagonal output keep one CTA per tile (no diagonal in the split form)
   int tile = 0;  // 0: BM x BN, 1: BM x BN_NARROW (no ring mode, no diagonal)
   if (force_splitk > 0) {
@@ -976,7 +970,7 @@ cudaError_t launch_minplus_gemm(const GemmParams& p, bool ring, cudaStream_t s, 
       S = t.p[0];
       tile = t.p[1];
     } else {
-      const GemmShape g = gemm_shape(p.M, p.N, p.K);
+      const GemmShape g = shape ? *shape : gemm_shape(p.M, p.N, p.K);
       S = g.S;
       tile = g.tile;
     }
@@ -1006,12 +1000,13 @@ cudaError_t launch_minplus_gemm(const GemmParams& p, bool ring, cudaStream_t s, 
 
 // The tensor-core launch of a product (not in ring mode, no diagonal), and the DPX launch for what it left.
 // Only a product whose modeled DPX schedule is kTcGain times the tensor cores' is tried: where the operands' values are
-// against it the look at a sample costs 4 us.  At the line (1.5 to 2): 700^3, 23 against 25 us, is left out; 1024^3, 25
-// against 43 (47 where the sample says no), is tried.  2048^3 takes 35 against 271, 4096^3 129 against 1946.
+// against it the look at a sample costs 4 us.  At the line (1.5 to 2): 700^3, 23 against 25 us, is left out; 1024^3, 23
+// against 43 (47 where the sample says no), is tried.  2048^3 takes 31 against 271, 4096^3 128 against 1946.
 constexpr double kTcGain = 1.8;
 cudaError_t launch_minplus_product(const GemmParams& p, cudaStream_t s) {
   bool marked = false;
   const tc::Code code = tc_code(p.K, p.lda, p.ldb);
+  const GemmShape shape = gemm_shape(p.M, p.N, p.K);
   if (code.L) {
     const int64_t pairs = sm_count() / 2, gy = (p.M + 2 * BM - 1) / (2 * BM), KT = (p.K + tc::kBK - 1) / tc::kBK;
     // the width with the shorter schedule: rounds of the pairs x clocks of one tile
@@ -1022,7 +1017,7 @@ cudaError_t launch_minplus_product(const GemmParams& p, cudaStream_t s) {
       const int64_t cost = (x * gy + pairs - 1) / pairs * (h == 1 ? 1080 * KT + 9000 : 1540 * KT + 14000);
       if (h == 1 || cost < best) best = cost, nh = h, gx = x;
     }
-    if (gemm_shape(p.M, p.N, p.K).clocks > kTcGain * (double)(best + 16000)) {
+    if (shape.clocks > kTcGain * (double)(best + 16000)) {
       const int64_t n = gx * gy < pairs ? gx * gy : pairs;
       const cudaError_t e =
           nh == 1 ? launch_kernel<minplus_tc_kernel<1>>(dim3((unsigned)(2 * n)), tc::kThreads, tc::smem_bytes(1), 1,
@@ -1033,7 +1028,7 @@ cudaError_t launch_minplus_product(const GemmParams& p, cudaStream_t s) {
       marked = true;
     }
   }
-  return launch_minplus_gemm(p, false, s, 0, 0, marked);
+  return launch_minplus_gemm(p, false, s, 0, 0, marked, &shape);
 }
 
 }  // namespace rd

@@ -88,12 +88,20 @@ struct GemmParams {
   int slots;
 };
 
+// The built-in launch shape of a DPX product: the tile (0: 128 x 256, 1: 128 x 128), the number of K slices S, and the
+// modeled clocks.
+struct GemmShape {
+  int S, tile;
+  double clocks;
+};
+
 // Launchers implemented in the .cu files.
 // force_splitk > 0 (not in ring mode): split K by exactly that factor, with tile shape force_tile (0: 128 x
 // 256, 1: 128 x 128) -- the autotuner's trials; else the tuning table's factor and tile for the product's
-// size class, else the built-in rule (the wide tile).
+// size class, else the modeled shape (`shape`, where the caller has it).  marked: only the tiles that the tensor-core
+// launch before it has marked.
 cudaError_t launch_minplus_gemm(const GemmParams& p, bool ring, cudaStream_t s, int force_splitk = 0,
-                                int force_tile = 0, bool marked = false);
+                                int force_tile = 0, bool marked = false, const GemmShape* shape = nullptr);
 bool splitk_suits(int S, int64_t K);         // S in {1, 2, 4, 8} and every K slice non-empty
 int64_t gemm_tiles(int64_t M, int64_t N);  // output tiles (CTAs of an unsplit launch)
 
