@@ -459,6 +459,10 @@ __device__ __forceinline__ void tc_finish(const GemmParams& p, bool ok, int64_t 
   }
 #pragma unroll
   for (int h = 0; h < NH; ++h) {
+    if (threadIdx.x == 0 && m0 < p.M && n0 + h * BN < p.N) {
+      tc::count(skip[h] ? &tc::Check::left : &tc::Check::decided, 1);
+      if (!skip[h]) tc::count(&tc::Check::fixed, s->cnt[h]);
+    }
     if (skip[h]) {
       if (threadIdx.x == 0) mark_tile(p, m0, n0 + h * BN);
     } else if (s->cnt[h] > 0) {
@@ -499,9 +503,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc::kThreads, 1)
     int64_t tm, tn;
     grouped_tile(t, gx, gy, &tm, &tn);
     const int64_t m0 = (tm * 2 + rank) * BM, n0 = tn * NH * BN;
-    const bool ok = tc::tile<NH>(p, m0, n0, code, buf, &ts, pr);
+    const bool ok = tc::usable(&ts, pr) && tc::tile<NH>(p, m0, n0, code, buf, &ts, pr);
     if (threadIdx.x < tc::kProducers) tc_finish<NH>(p, ok, m0, n0, buf, &ts);
   }
+  if (threadIdx.x == 0 && tc::cta_rank() == 0 && !tc::usable(&ts, pr)) tc::count(&tc::Check::lost, 1);
   tc::close<NH>(&ts);
 }
 
@@ -721,12 +726,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc::kThreads, 1)
       __syncthreads();
     }
     if (worth) {
-      const bool ok = tc::tile<NH>(p, at[0], at[1], code, buf, &ts, pr);
+      const bool ok = tc::usable(&ts, pr) && tc::tile<NH>(p, at[0], at[1], code, buf, &ts, pr);
       if (threadIdx.x < tc::kProducers) tc_finish<NH>(p, ok, at[0], at[1], buf, &ts);
     } else if (threadIdx.x < NH) {
       mark_tile(p, at[0], at[1] + threadIdx.x * BN);
     }
   }
+  if (threadIdx.x == 0 && tc::cta_rank() == 0 && !tc::usable(&ts, pr)) tc::count(&tc::Check::lost, 1);
   tc::close<NH>(&ts);
 }
 
@@ -1355,3 +1361,20 @@ extern "C" rd_status rd_minplus_gemm_batched(const rd_gemm_problem* problems, in
   if (e != cudaSuccess) { set_cuda_error(e); return RD_ERR_CUDA; }
   return RD_OK;
 }
+
+#ifdef RD_CHECKED
+// The checked build's access to the tensor-core tile's settings and counts, for the tests: sets wait_rounds, hold_at
+// and hold_us as given (null: none), returns the counts since the last call and clears them.  Synchronous.
+extern "C" rd_status rd_tc_check(const uint32_t* settings, uint32_t* counts) {
+  tc::Check c;
+  cudaError_t e = cudaMemcpyFromSymbol(&c, tc::g_check, sizeof(c));
+  if (e == cudaSuccess) {
+    if (counts) counts[0] = c.decided, counts[1] = c.fixed, counts[2] = c.left, counts[3] = c.lost;
+    if (settings) c.wait_rounds = settings[0], c.hold_at = (int32_t)settings[1], c.hold_us = settings[2];
+    c.decided = c.fixed = c.left = c.lost = 0;
+    e = cudaMemcpyToSymbol(tc::g_check, &c, sizeof(c));
+  }
+  if (e != cudaSuccess) { set_cuda_error(e); return RD_ERR_CUDA; }
+  return RD_OK;
+}
+#endif

@@ -41,6 +41,29 @@ constexpr int64_t kMaxLd = 1 << 23;                                   // strides
 constexpr int64_t kMinK = 64, kMaxK = (int64_t)1 << 19;
 constexpr uint32_t kWaitRounds = 1u << 18;                            // bound of every mbarrier wait
 
+// Checked builds (-DRD_CHECKED): what rd_tc_check sets and reads.  Every launch reads the settings and adds to the
+// counts.
+struct Check {
+  uint32_t wait_rounds;  // bound of the waits of a tile (those before the shared memory is given up keep kWaitRounds)
+  int32_t hold_at;       // the first pair's MMA warp pauses before this stage, counted from 0 over its tiles (-1: never)
+  uint32_t hold_us;      // for so many microseconds, as a warp that is kept from running would
+  uint32_t decided, fixed, left, lost;  // parts of C written, outputs computed term by term, parts left to the DPX
+                                        // launch, pairs of CTAs that lost their pipeline
+};
+#ifdef RD_CHECKED
+__device__ Check g_check = {kWaitRounds, -1, 0, 0, 0, 0, 0};
+__device__ __forceinline__ uint32_t wait_rounds() { return *(volatile uint32_t*)&g_check.wait_rounds; }
+__device__ __forceinline__ void count(uint32_t Check::*what, uint32_t n) { atomicAdd(&(g_check.*what), n); }
+__device__ __forceinline__ void hold(uint32_t stage) {
+  if (blockIdx.x > 1 || (int32_t)stage != *(volatile int32_t*)&g_check.hold_at) return;
+  for (uint32_t us = *(volatile uint32_t*)&g_check.hold_us; us > 0; --us) __nanosleep(1000);
+}
+#else
+__device__ __forceinline__ constexpr uint32_t wait_rounds() { return kWaitRounds; }
+__device__ __forceinline__ void count(uint32_t Check::*, uint32_t) {}
+__device__ __forceinline__ void hold(uint32_t) {}
+#endif
+
 // Window and exponent step for sums of at most K terms: 2^(L-1) >= K, and the largest W for which 2^(L-1)
 // products of two level-0 codes stay below 2^127: 2 (L W - 127) + L - 1 <= 126.
 struct Code {
@@ -60,7 +83,8 @@ struct Shared {
   uint64_t all;       // every MMA issued so far is done
   int64_t at[2];      // the tile's m0 and n0
   uint32_t tmem;      // the accumulator's TMEM address
-  uint32_t bad;       // an operand outside the documented range in either CTA, or a wait that ran out
+  uint32_t bad;       // an operand outside the documented range in either CTA
+  uint32_t lost[2];   // a wait ran out in either CTA, in an even or an odd phase of `all`; stays set
   uint32_t look[2];   // the early look: undecided outputs and outputs looked at, both CTAs
   uint32_t na, nb;    // the sample's counts
   uint32_t cnt[2];    // undecided outputs of each 128 x 256 part
@@ -70,7 +94,7 @@ struct Shared {
 // Progress of the pipeline, carried across the tiles that a pair works on.
 struct Progress {
   uint32_t st = 0, round = 0;  // next stage, and how often the ring has gone round
-  uint32_t all = 0;            // completed phases of `all`
+  uint32_t all = 0;            // phases of `all` so far
 };
 
 __device__ __forceinline__ uint32_t sm_u32(const void* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
@@ -95,19 +119,25 @@ __device__ __forceinline__ void add_at(uint32_t addr, uint32_t v) {
 __device__ __forceinline__ void mbar_init(uint64_t* b, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(sm_u32(b)), "r"(count) : "memory");
 }
-__device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity) {
-  for (uint32_t n = 0; n < kWaitRounds; ++n) {
-    uint32_t done;
-    asm volatile(
-        "{\n.reg .pred p;\n"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-        "selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(done)
-        : "r"(sm_u32(b)), "r"(parity)
-        : "memory");
-    if (done) return true;
+__device__ __forceinline__ bool mbar_try(uint64_t* b, uint32_t parity) {
+  uint32_t done;
+  asm volatile(
+      "{\n.reg .pred p;\n"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+      "selp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(done)
+      : "r"(sm_u32(b)), "r"(parity)
+      : "memory");
+  return done;
+}
+// A wait of phase `all` of the pipeline.  Running out, or finding that another wait has, is reported to both CTAs.
+__device__ __forceinline__ void pipe_wait(Shared* s, uint64_t* b, uint32_t parity, uint32_t all) {
+  for (uint32_t n = 0; !mbar_try(b, parity); ++n) {
+    if (n < 64 || (n < wait_rounds() && !(*(volatile uint32_t*)&s->lost[0] | *(volatile uint32_t*)&s->lost[1]))) continue;
+    add_at(at_rank(&s->lost[all & 1], 0), 1);
+    add_at(at_rank(&s->lost[all & 1], 1), 1);
+    break;
   }
-  return false;
 }
 // On a barrier of either CTA.  What the arriving warp stored is read by the tensor core alone, each CTA's by its own:
 // the proxy fence before the arrival orders that, so the release stays at CTA scope.  (At cluster scope it waits for
@@ -126,6 +156,7 @@ __device__ __forceinline__ void open(Shared* s) {
       mbar_init(&s->empty[i], 1);
     }
     mbar_init(&s->all, 1);
+    s->lost[0] = s->lost[1] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (threadIdx.x < 32) {
@@ -265,7 +296,6 @@ struct Feed {
   uint32_t w2, step, top2;  // W in both halves; one level in a bf16's bits; level 0 (level W is the code 0)
   uint32_t seen, seen_b[4]; // the bits of all entries; of B's per word where N cuts the chunk
   Progress pr;
-  bool ok;
 };
 __device__ __forceinline__ uint4 encode(const Feed& f, const uint4& v) {
   return make_uint4(f.top2 - __vminu2(v.x, f.w2) * f.step, f.top2 - __vminu2(v.y, f.w2) * f.step,
@@ -282,7 +312,7 @@ struct Chunks {
 };
 template <int NH>
 __device__ __forceinline__ void stage_free(Feed& f, Shared* s) {  // the MMAs that read the next stage are done
-  if (f.pr.round > 0) f.ok &= mbar_wait(&s->empty[f.pr.st], (f.pr.round - 1) & 1);
+  if (f.pr.round > 0) pipe_wait(s, &s->empty[f.pr.st], (f.pr.round - 1) & 1, f.pr.all);
 }
 template <int NH>
 __device__ __forceinline__ void stage_done(Feed& f) {
@@ -335,6 +365,14 @@ __device__ __forceinline__ void feed(Feed& f, Shared* s, const int n) {
   put(false);
 }
 
+// A wait ran out in phase `all` - 1 or before: read behind that phase's cluster barrier, and the same in all threads of
+// both CTAs, because the next write to the same slot lies behind the next phase's barrier.
+__device__ __forceinline__ bool lost_by(const Shared* s, uint32_t all) {
+  return *(volatile const uint32_t*)&s->lost[(all - 1) & 1];
+}
+// Whether the pair's pipeline is intact after its tiles so far.
+__device__ __forceinline__ bool usable(const Shared* s, const Progress& pr) { return pr.all == 0 || !lost_by(s, pr.all); }
+
 // The pair's tile at (m0, n0) -- m0 is this CTA's first row, n0 the tile's first column -- over all K terms.  On true,
 // this CTA's 128 x 256 NH outputs are in shared memory at buf: row r, 16-byte vector c (columns 8c ..) at
 // T[r 32 NH + (c ^ (r & 7))], undecided outputs as RD_INF, those inside M x N counted per 256 columns in s->cnt and the
@@ -342,6 +380,10 @@ __device__ __forceinline__ void feed(Feed& f, Shared* s, const int n) {
 // documented range, a wait that ran out, or too little decided: an eighth of the way some of the outputs are
 // looked at).  Called by all threads of both CTAs with the same answer; the caller syncs the producers before the
 // next call.
+//
+// A wait that runs out leaves the two CTAs' stages and barrier phases out of step with each other, for good: what was
+// waited for may still come.  So it ends the tensor cores' part in this pair (usable): this tile and all later ones are
+// the DPX kernel's, no thread waits for long again, and the MMAs already issued are waited for.
 template <int NH>
 __device__ __forceinline__ bool tile(const GemmParams& p, const int64_t m0, const int64_t n0, const Code code, char* buf,
                                      Shared* s, Progress& pr) {
@@ -357,9 +399,9 @@ __device__ __forceinline__ bool tile(const GemmParams& p, const int64_t m0, cons
   if (tid == 0) s->bad = s->look[0] = s->look[1] = s->cnt[0] = s->cnt[1] = 0;
   // whether the early look leaves the tile to the DPX kernel: a share f left open by an eighth of the terms is f^8 at
   // the end, 64 of 32768 at f = 0.46
-  auto hopeless = [&]() {
+  auto hopeless = [&](uint32_t all) {
     cluster_sync();  // both CTAs' counts are in
-    const bool r = (float)s->look[0] > 0.46f * (float)s->look[1];
+    const bool r = (float)s->look[0] > 0.46f * (float)s->look[1] || lost_by(s, all);
     cluster_sync();  // and read
     return r;
   };
@@ -376,15 +418,15 @@ __device__ __forceinline__ bool tile(const GemmParams& p, const int64_t m0, cons
                                 ((uint32_t)((2 * kBM) >> 4) << 24);
     const uint32_t base = sm_u32(buf), tmem = s->tmem;
     const bool issuer = rank == 0 && lane == 0;
-    bool ok = true;
     for (int kt = 0; kt < KT; ++kt) {
       if (kt == check) {
         if (issuer) commit(&s->all);
         __syncwarp();
-        if (hopeless()) return false;
+        if (hopeless(++pr.all)) return false;
       }
       if (rank == 0) {
-        ok &= mbar_wait(&s->full[pr.st], pr.round & 1);
+        hold(pr.round * stages(NH) + pr.st);
+        pipe_wait(s, &s->full[pr.st], pr.round & 1, pr.all);
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         if (issuer) {
           const uint32_t a0 = base + pr.st * stage_bytes(NH), b0 = a0 + kBytesA;
@@ -401,10 +443,7 @@ __device__ __forceinline__ bool tile(const GemmParams& p, const int64_t m0, cons
       if (++pr.st == stages(NH)) pr.st = 0, ++pr.round;
     }
     if (issuer) commit(&s->all);
-    if (!ok && lane == 0) {
-      add_at(at_rank(&s->bad, 0), 1);
-      add_at(at_rank(&s->bad, 1), 1);
-    }
+    ++pr.all;
     __syncwarp();
     cluster_sync();
     return false;
@@ -435,7 +474,6 @@ __device__ __forceinline__ bool tile(const GemmParams& p, const int64_t m0, cons
   f.top2 = (code.L * code.W << 7) * 0x00010001u;
   f.seen = f.seen_b[0] = f.seen_b[1] = f.seen_b[2] = f.seen_b[3] = 0;
   f.pr = pr;
-  f.ok = true;
   // the stage of the last terms: RD_INF in A from K on
   auto feed_last = [&](int kt) {
     uint4 ra[NA], rb[NB];
@@ -469,9 +507,13 @@ __device__ __forceinline__ bool tile(const GemmParams& p, const int64_t m0, cons
     stage_done<NH>(f);
   };
   auto drain = [&]() {  // every MMA issued so far is complete
-    f.ok &= mbar_wait(&s->all, f.pr.all & 1);
+    pipe_wait(s, &s->all, f.pr.all & 1, f.pr.all);
     ++f.pr.all;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  };
+  // Behind the cluster barrier after a drain: the MMA warp has issued all it will.  None is in flight afterwards.
+  auto settle = [&]() {
+    for (uint32_t n = 0; n < kWaitRounds && !mbar_try(&s->all, (f.pr.all - 1) & 1); ++n) {}
   };
   // What the accumulator is read with, computed anew where it is needed: held across the loop it cost spills there.
   struct Reader {
@@ -511,7 +553,7 @@ __device__ __forceinline__ bool tile(const GemmParams& p, const int64_t m0, cons
       add_at(at_rank(&s->look[1], lane), seen_n);
     }
     __syncwarp();
-    return hopeless();
+    return hopeless(f.pr.all);
   };
   // whole stages, short of the row of B that no row follows where N cuts a chunk
   const int inside = (int)((p.N & 7) != 0 ? (p.K - 1) / kBK : p.K / kBK);
@@ -526,6 +568,7 @@ __device__ __forceinline__ bool tile(const GemmParams& p, const int64_t m0, cons
     for (; kt < stop; ++kt) feed_last(kt);
     if (stop == KT) break;
     if (look()) {
+      if (lost_by(s, f.pr.all)) settle();
       pr = f.pr;
       return false;
     }
@@ -534,11 +577,15 @@ __device__ __forceinline__ bool tile(const GemmParams& p, const int64_t m0, cons
   for (int e = 0; e < 8; ++e)
     if (e < cut) f.seen |= f.seen_b[e >> 1] & (0xFFFFu << (16 * (e & 1)));
   drain();
-  const bool wrong = __any_sync(0xFFFFFFFFu, (f.seen & 0xC000C000u) != 0 || !f.ok);
+  const bool wrong = __any_sync(0xFFFFFFFFu, (f.seen & 0xC000C000u) != 0);
   pr = f.pr;
   if (wrong && lane < 2) add_at(at_rank(&s->bad, lane), 1);
   __syncwarp();
   cluster_sync();  // both CTAs' flags are in; nobody reads a stage any more
+  if (lost_by(s, f.pr.all)) {
+    settle();
+    return false;
+  }
   if (s->bad) return false;
 
   const Reader at(p, s);

@@ -1,0 +1,112 @@
+"""Cases of the tensor-core tile that need the checked build of the library (librd_checked.so, -DRD_CHECKED): a wait
+that runs out, and which path computed a product.
+
+Not collected by a plain `pytest tests` (the file name does not start with test_): test_gpu_tc_checked.py runs it in a
+child process.
+"""
+import ctypes
+import os
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+INF = 0x3FFF
+
+
+@pytest.fixture(scope="module")
+def rd():
+    lib = os.environ.get("RD_CHECKED_LIB")
+    if not lib:
+        pytest.fail("run by test_gpu_tc_checked.py under the checked build")
+    import paper_2409_17658_gb300 as rd
+
+    prev = rd.use_library(lib)
+    yield rd
+    rd.use_library_handle(prev)
+
+
+def check(rd, wait_rounds=1 << 18, hold_at=-1, hold_us=0):
+    """Applies settings (by default: the ordinary ones); returns the counts since the last call."""
+    settings, counts = (ctypes.c_uint32 * 3)(wait_rounds, hold_at & 0xFFFFFFFF, hold_us), (ctypes.c_uint32 * 4)()
+    assert rd._lib().rd_tc_check(settings, counts) == rd.RD_OK
+    return dict(zip(("decided", "fixed", "left", "lost"), counts))
+
+
+@pytest.fixture(autouse=True)
+def ordinary_settings(rd):
+    check(rd)
+    yield
+    check(rd)
+
+
+def draw(rows, cols, top, inf, seed):
+    r = np.random.default_rng(seed)
+    return np.where(r.random((rows, cols)) < inf, INF, r.integers(0, top, (rows, cols))).astype(np.int16)
+
+
+def upload(host):
+    import torch
+
+    t = torch.full((host.shape[0], (host.shape[1] + 7) // 8 * 8), -3, dtype=torch.int16)
+    t[:, :host.shape[1]] = torch.from_numpy(host)
+    return t.cuda()
+
+
+def result(M, N):
+    import torch
+
+    return torch.full((M, (N + 7) // 8 * 8), -7, dtype=torch.int16, device="cuda")
+
+
+def assert_product(orc, a, b, C, seed=1):
+    """Sampled entries, and the last row and column, against the oracle."""
+    M, N = a.shape[0], b.shape[1]
+    r = np.random.default_rng(seed)
+    ri = np.concatenate([r.integers(0, M, 20000), np.full(N, M - 1), np.arange(M)])
+    cj = np.concatenate([r.integers(0, N, 20000), np.arange(N), np.full(M, N - 1)])
+    got = C.cpu().numpy()
+    assert np.array_equal(got[ri, cj].astype(np.int32), orc.minplus_i16_entries(a, b, ri, cj))
+    assert (got[:, N:] == -7).all()
+
+
+def parts(M, N):
+    return -(-M // 128) * -(-N // 256)
+
+
+# (M, N, K) and the stage of a tile: tiles of 256 columns, three for the pair that is held; tiles of 512, two; the same
+# with an early look behind that stage
+LOST = [(256 * 76 * 2 + 300, 250, 600, 5), (256 * 30, 2500, 700, 5), (256 * 30, 2500, 2600, 2)]
+
+
+@pytest.mark.parametrize("tile", [0, 1])
+@pytest.mark.parametrize("M,N,K,stage", LOST)
+def test_a_wait_that_runs_out_leaves_the_rest_of_the_pair(rd, orc, M, N, K, stage, tile):
+    """The held pair's MMA warp comes back after every other thread has given up; its tiles from that one on are the
+    DPX launch's, the others' are not, and the next product finds nothing changed."""
+    a, b = draw(M, K, 4, 0.1, 1), draw(K, N, 4, 0.1, 2)
+    A, B, C = upload(a), upload(b), result(M, N)
+    check(rd, wait_rounds=256, hold_at=tile * -(-K // 64) + stage, hold_us=100_000)
+    rd.minplus_gemm(A, B, C, M, N, K)
+    seen = check(rd)
+    assert seen["lost"] == 1 and seen["left"] >= 2 and seen["decided"] + seen["left"] == parts(M, N), seen
+    assert_product(orc, a, b, C)
+    C.fill_(-7)
+    rd.minplus_gemm(A, B, C, M, N, K)
+    seen = check(rd)
+    assert seen == dict(decided=parts(M, N), fixed=seen["fixed"], left=0, lost=0), seen
+    assert_product(orc, a, b, C)
+
+
+def test_a_wait_that_runs_out_in_a_batch(rd, orc):
+    shapes = [(256 * 20, 2000, 640), (3000, 3001, 600), (700, 520, 200)]
+    host = [(draw(M, K, 4, 0.1, i), draw(K, N, 4, 0.1, 9 + i)) for i, (M, N, K) in enumerate(shapes)]
+    problems = [(upload(a), upload(b), result(M, N), M, N, K, None) for (a, b), (M, N, K) in zip(host, shapes)]
+    check(rd, wait_rounds=256, hold_at=3, hold_us=100_000)
+    rd.minplus_gemm_batched(problems)
+    seen = check(rd)
+    total = sum(parts(M, N) for M, N, _ in shapes)
+    assert seen["lost"] == 1 and seen["left"] >= 2 and seen["decided"] + seen["left"] == total, seen
+    for (a, b), p in zip(host, problems):
+        assert_product(orc, a, b, p[2])
