@@ -491,13 +491,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc::kThreads, 1)
   extern __shared__ __align__(16) char tc_smem[];
   __shared__ tc::Shared ts;
   const int64_t rank = tc::cta_rank(), pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
-  if (!tc::worth(p, code.W, &ts)) {
-    for (int64_t t = pair + threadIdx.x * pairs; t < gx * gy; t += tc::kThreads * pairs)
-      for (int h = 0; h < NH; ++h) mark_tile(p, (t / gx * 2 + rank) * BM, (t % gx * NH + h) * BN);
+  tc::open<NH>(&ts);
+  if (!tc::worth<true>(p, code.W, &ts, 0)) {
+    for (int64_t t = pair + threadIdx.x * pairs; t < gx * gy; t += tc::kThreads * pairs) {
+      int64_t tm, tn;
+      grouped_tile(t, gx, gy, &tm, &tn);
+      for (int h = 0; h < NH; ++h) mark_tile(p, (tm * 2 + rank) * BM, (tn * NH + h) * BN);
+    }
     return;
   }
   char* buf = tc_buffer(tc_smem);
-  tc::open<NH>(&ts);
+  tc::take_accumulator<NH>(&ts);
   tc::Progress pr;
   for (int64_t t = pair; t < gx * gy; t += pairs) {
     int64_t tm, tn;
@@ -693,7 +697,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc::kThreads, 1)
   char* buf = tc_buffer(tc_smem);
   if (threadIdx.x == 0) cur = -1;
   tc::open<NH>(&ts);
+  tc::cluster_wait();
+  tc::take_accumulator<NH>(&ts);
   tc::Progress pr;
+  uint32_t turn = 0;
 #pragma unroll 1
   for (int64_t t = blockIdx.x >> 1; t < bp.tc_start[bp.count]; t += gridDim.x >> 1) {
     __syncthreads();  // everybody is done with the previous tile
@@ -721,7 +728,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc::kThreads, 1)
     }
     __syncthreads();
     if (changed) {
-      const bool w = tc::worth(p, code.W, &ts);
+      const bool w = tc::worth<false>(p, code.W, &ts, turn++);
       if (threadIdx.x == 0) worth = w;
       __syncthreads();
     }
@@ -1363,14 +1370,14 @@ extern "C" rd_status rd_minplus_gemm_batched(const rd_gemm_problem* problems, in
 }
 
 #ifdef RD_CHECKED
-// The checked build's access to the tensor-core tile's settings and counts, for the tests: sets wait_rounds, hold_at
-// and hold_us as given (null: none), returns the counts since the last call and clears them.  Synchronous.
+// The checked build's access to the tensor-core tile's settings and counts, for the tests: sets wait_rounds, hold_at,
+// hold_us and deaf as given (null: none), returns the counts since the last call and clears them.  Synchronous.
 extern "C" rd_status rd_tc_check(const uint32_t* settings, uint32_t* counts) {
   tc::Check c;
   cudaError_t e = cudaMemcpyFromSymbol(&c, tc::g_check, sizeof(c));
   if (e == cudaSuccess) {
     if (counts) counts[0] = c.decided, counts[1] = c.fixed, counts[2] = c.left, counts[3] = c.lost;
-    if (settings) c.wait_rounds = settings[0], c.hold_at = (int32_t)settings[1], c.hold_us = settings[2];
+    if (settings) c.wait_rounds = settings[0], c.hold_at = (int32_t)settings[1], c.hold_us = settings[2], c.deaf = settings[3];
     c.decided = c.fixed = c.left = c.lost = 0;
     e = cudaMemcpyToSymbol(tc::g_check, &c, sizeof(c));
   }

@@ -47,21 +47,24 @@ struct Check {
   uint32_t wait_rounds;  // bound of the waits of a tile (those before the shared memory is given up keep kWaitRounds)
   int32_t hold_at;       // the first pair's MMA warp pauses before this stage, counted from 0 over its tiles (-1: never)
   uint32_t hold_us;      // for so many microseconds, as a warp that is kept from running would
+  uint32_t deaf;         // bit r: CTA r of a pair finds nothing in its half of the sample, whatever it holds
   uint32_t decided, fixed, left, lost;  // parts of C written, outputs computed term by term, parts left to the DPX
                                         // launch, pairs of CTAs that lost their pipeline
 };
 #ifdef RD_CHECKED
-__device__ Check g_check = {kWaitRounds, -1, 0, 0, 0, 0, 0};
+__device__ Check g_check = {kWaitRounds, -1, 0, 0, 0, 0, 0, 0};
 __device__ __forceinline__ uint32_t wait_rounds() { return *(volatile uint32_t*)&g_check.wait_rounds; }
 __device__ __forceinline__ void count(uint32_t Check::*what, uint32_t n) { atomicAdd(&(g_check.*what), n); }
 __device__ __forceinline__ void hold(uint32_t stage) {
   if (blockIdx.x > 1 || (int32_t)stage != *(volatile int32_t*)&g_check.hold_at) return;
   for (uint32_t us = *(volatile uint32_t*)&g_check.hold_us; us > 0; --us) __nanosleep(1000);
 }
+__device__ __forceinline__ bool deaf(uint32_t rank) { return *(volatile uint32_t*)&g_check.deaf >> rank & 1; }
 #else
 __device__ __forceinline__ constexpr uint32_t wait_rounds() { return kWaitRounds; }
 __device__ __forceinline__ void count(uint32_t Check::*, uint32_t) {}
 __device__ __forceinline__ void hold(uint32_t) {}
+__device__ __forceinline__ constexpr bool deaf(uint32_t) { return false; }
 #endif
 
 // Window and exponent step for sums of at most K terms: 2^(L-1) >= K, and the largest W for which 2^(L-1)
@@ -86,7 +89,7 @@ struct Shared {
   uint32_t bad;       // an operand outside the documented range in either CTA
   uint32_t lost[2];   // a wait ran out in either CTA, in an even or an odd phase of `all`; stays set
   uint32_t look[2];   // the early look: undecided outputs and outputs looked at, both CTAs
-  uint32_t na, nb;    // the sample's counts
+  uint32_t vote[3][2];  // the sample's counts over both CTAs, one slot per question in turn
   uint32_t cnt[2];    // undecided outputs of each 128 x 256 part
   uint32_t list[2][kMostFix];
 };
@@ -108,8 +111,11 @@ __device__ __forceinline__ uint32_t at_rank(const void* p, uint32_t rank) {  // 
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(sm_u32(p)), "r"(rank));
   return a;
 }
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
+  cluster_arrive();
+  cluster_wait();
 }
 __device__ __forceinline__ void producers_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kProducers) : "memory"); }
 __device__ __forceinline__ void add_at(uint32_t addr, uint32_t v) {
@@ -146,7 +152,8 @@ __device__ __forceinline__ void arrive_at(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
-// Once per CTA, all threads of the pair: the barriers and the accumulator's TMEM columns.
+// Once per CTA, all threads of the pair: first the barriers, with an arrival at the cluster barrier (behind whose wait
+// the other CTA has started and its barriers are ready), later the accumulator's TMEM columns.
 template <int NH>
 __device__ __forceinline__ void open(Shared* s) {
   if (threadIdx.x == 0) {
@@ -157,8 +164,13 @@ __device__ __forceinline__ void open(Shared* s) {
     }
     mbar_init(&s->all, 1);
     s->lost[0] = s->lost[1] = 0;
+    s->vote[0][0] = s->vote[0][1] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  cluster_arrive();
+}
+template <int NH>
+__device__ __forceinline__ void take_accumulator(Shared* s) {
   if (threadIdx.x < 32) {
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(sm_u32(&s->tmem)),
                  "n"(NH * kBN)
@@ -166,7 +178,7 @@ __device__ __forceinline__ void open(Shared* s) {
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  cluster_sync();
+  __syncthreads();  // the other CTA's columns are taken before its first stages are
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 // After the last tile, all threads of the pair; no MMA is in flight then.
@@ -239,17 +251,18 @@ __device__ __forceinline__ uint4 row8(const int16_t* row, int64_t e0, int64_t le
 // Whether a product is worth trying: 256 vectors of 8 entries of each operand, spread over it, give the shares pa,
 // pb of entries below W; with K pa pb / 2 pairs expected to sum to at most W an output stays undecided with
 // probability exp(-K pa pb / 2), and a part of 32768 outputs needs nearly all of them decided.  Only speed hangs on
-// this.  Every CTA reads the same entries and gets the same answer.  All threads call it; one load of each
-// operand per thread, so it costs one memory latency.
-__device__ __forceinline__ bool worth(const GemmParams& p, uint32_t W, Shared* s) {
+// this, as long as both CTAs of a pair get the same answer: each reads half of the sample and adds what it finds to the
+// counts of both, so the answer is the same whatever the loads return.  All threads of the pair call it, for the
+// turn-th time; one load of each operand per thread, so it costs one memory latency.  FIRST: right behind open().
+template <bool FIRST>
+__device__ __forceinline__ bool worth(const GemmParams& p, uint32_t W, Shared* s, uint32_t turn) {
   const int tid = threadIdx.x;
-  if (tid == 0) s->na = s->nb = 0;
   const uint4 none = make_uint4(kInf2, kInf2, kInf2, kInf2);
   uint4 va = none, vb = none;
-  if (tid < 256) {
-    const int spread = (tid & 15) * 16 + (tid >> 4);
-    const int64_t ra = (tid * p.M) >> 8, ca = ((spread * p.K) >> 8) & ~(int64_t)7;
-    const int64_t rb = (tid * p.K) >> 8, cb = ((spread * p.N) >> 8) & ~(int64_t)7;
+  if (tid < 128) {
+    const int i = tid + 128 * (int)cta_rank(), spread = (i & 15) * 16 + (i >> 4);
+    const int64_t ra = (i * p.M) >> 8, ca = ((spread * p.K) >> 8) & ~(int64_t)7;
+    const int64_t rb = (i * p.K) >> 8, cb = ((spread * p.N) >> 8) & ~(int64_t)7;
     if (ca + 8 <= p.K) va = __ldg(reinterpret_cast<const uint4*>(p.A + ra * p.lda + ca));
     if (cb + 8 <= p.N) vb = __ldg(reinterpret_cast<const uint4*>(p.B + rb * p.ldb + cb));
   }
@@ -260,14 +273,16 @@ __device__ __forceinline__ bool worth(const GemmParams& p, uint32_t W, Shared* s
   };
   const int na = __reduce_add_sync(0xFFFFFFFFu, below(va));
   const int nb = __reduce_add_sync(0xFFFFFFFFu, below(vb));
-  __syncthreads();
-  if ((tid & 31) == 0) {
-    atomicAdd(&s->na, (uint32_t)na);
-    atomicAdd(&s->nb, (uint32_t)nb);
+  const uint32_t slot = turn % 3;
+  uint32_t* next = s->vote[(turn + 1) % 3];  // last read two questions ago, before the barrier of the one in between
+  if (tid == 0) next[0] = next[1] = 0;
+  if (FIRST) cluster_wait();
+  if (tid < 128 && (tid & 31) < 2 && !deaf(cta_rank())) {
+    add_at(at_rank(&s->vote[slot][0], tid & 1), (uint32_t)na);
+    add_at(at_rank(&s->vote[slot][1], tid & 1), (uint32_t)nb);
   }
-  __syncthreads();
-  const float pa = (float)s->na * (1.f / 2048.f), pb = (float)s->nb * (1.f / 2048.f);
-  __syncthreads();  // the counts are read before the next use
+  cluster_sync();
+  const float pa = (float)s->vote[slot][0] * (1.f / 2048.f), pb = (float)s->vote[slot][1] * (1.f / 2048.f);
   return (float)p.K * pa * pb * 0.5f >= 6.2f;  // 32768 exp(-6.2) = 66 undecided outputs
 }
 

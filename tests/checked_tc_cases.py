@@ -27,9 +27,10 @@ def rd():
     rd.use_library_handle(prev)
 
 
-def check(rd, wait_rounds=1 << 18, hold_at=-1, hold_us=0):
+def check(rd, wait_rounds=1 << 18, hold_at=-1, hold_us=0, deaf=0):
     """Applies settings (by default: the ordinary ones); returns the counts since the last call."""
-    settings, counts = (ctypes.c_uint32 * 3)(wait_rounds, hold_at & 0xFFFFFFFF, hold_us), (ctypes.c_uint32 * 4)()
+    settings = (ctypes.c_uint32 * 4)(wait_rounds, hold_at & 0xFFFFFFFF, hold_us, deaf)
+    counts = (ctypes.c_uint32 * 4)()
     assert rd._lib().rd_tc_check(settings, counts) == rd.RD_OK
     return dict(zip(("decided", "fixed", "left", "lost"), counts))
 
@@ -110,3 +111,43 @@ def test_a_wait_that_runs_out_in_a_batch(rd, orc):
     assert seen["lost"] == 1 and seen["left"] >= 2 and seen["decided"] + seen["left"] == total, seen
     for (a, b), p in zip(host, problems):
         assert_product(orc, a, b, p[2])
+
+
+@pytest.mark.parametrize("batched", [False, True])
+@pytest.mark.parametrize("deaf", [1, 2, 3])
+def test_both_ctas_of_a_pair_go_by_one_answer(rd, orc, deaf, batched):
+    """One CTA of every pair finds nothing in its half of the sample, the other everything: both take the tensor cores
+    (their counts together still say so).  Neither finds anything: both leave every part."""
+    M, N, K = 2000, 1801, 1000
+    a, b = draw(M, K, 4, 0.1, 5), draw(K, N, 4, 0.1, 6)
+    A, B, C = upload(a), upload(b), result(M, N)
+    check(rd, deaf=deaf)
+    if batched:  # two products: the question is asked anew for each
+        C2 = result(M, N)
+        rd.minplus_gemm_batched([(A, B, C, M, N, K, None), (A, B, C2, M, N, K, None)])
+    else:
+        rd.minplus_gemm(A, B, C, M, N, K)
+    seen, n = check(rd), parts(M, N) * (2 if batched else 1)
+    assert (seen["decided"], seen["lost"]) == (0 if deaf == 3 else n, 0), seen
+    assert_product(orc, a, b, C)
+    if batched:
+        assert_product(orc, a, b, C2)
+
+
+@pytest.mark.parametrize("M,N,K", [(1300, 1000, 1100), (2000, 1801, 1000)])
+def test_operands_and_result_in_interleaved_rows(rd, orc, M, N, K):
+    """A, B and C side by side in the rows of one parent (row strides far above their widths)."""
+    import torch
+
+    ld = 2048
+    parent = torch.full((max(M, K), 3 * ld), -7, dtype=torch.int16)
+    a, b = draw(M, K, 33, 0.5, 7), draw(K, N, 33, 0.5, 8)
+    parent[:M, :K], parent[:K, ld:ld + N] = torch.from_numpy(a), torch.from_numpy(b)
+    parent = parent.cuda()
+    before, C = parent.clone(), parent[:M, 2 * ld:]
+    rd.minplus_gemm(parent[:M, :ld], parent[:K, ld:2 * ld], C, M, N, K)
+    seen = check(rd)
+    assert seen["decided"] == parts(M, N) and seen["left"] == 0, seen
+    assert_product(orc, a, b, C)
+    C[:, :N] = -7
+    assert torch.equal(parent, before)
