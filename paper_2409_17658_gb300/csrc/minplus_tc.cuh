@@ -172,6 +172,7 @@ __device__ __forceinline__ void open(Shared* s) {
 template <int NH>
 __device__ __forceinline__ void take_accumulator(Shared* s) {
   if (threadIdx.x < 32) {
+    __syncwarp();  // .aligned: the warp's lanes together, as in every tcgen05 instruction of a whole warp below
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(sm_u32(&s->tmem)),
                  "n"(NH * kBN)
                  : "memory");
@@ -187,6 +188,7 @@ __device__ __forceinline__ void close(Shared* s) {
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   cluster_sync();
   if (threadIdx.x < 32) {
+    __syncwarp();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(s->tmem), "n"(NH * kBN) : "memory");
   }
@@ -524,6 +526,7 @@ __device__ __forceinline__ bool tile(const GemmParams& p, const int64_t m0, cons
   auto drain = [&]() {  // every MMA issued so far is complete
     pipe_wait(s, &s->all, f.pr.all & 1, f.pr.all);
     ++f.pr.all;
+    __syncwarp();  // each lane has polled for itself
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   };
   // Behind the cluster barrier after a drain: the MMA warp has issued all it will.  None is in flight afterwards.
@@ -602,6 +605,7 @@ __device__ __forceinline__ bool tile(const GemmParams& p, const int64_t m0, cons
     return false;
   }
   if (s->bad) return false;
+  __syncwarp();
 
   const Reader at(p, s);
   const Decode level(code);
