@@ -487,16 +487,20 @@ __device__ __forceinline__ char* tc_buffer(char* smem) {
 // Pair c takes tiles c, c + pairs, ... of the gx x gy tiles of 256 x 256 NH in the grouped order.
 template <int NH>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc::kThreads, 1)
-    minplus_tc_kernel(GemmParams p, tc::Code code, int64_t gx, int64_t gy) {
+    minplus_tc_kernel(GemmParams p, tc::Code code, int64_t gx, int64_t gy, bool strict) {
   extern __shared__ __align__(16) char tc_smem[];
   __shared__ tc::Shared ts;
   const int64_t rank = tc::cta_rank(), pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
   tc::open<NH>(&ts);
-  if (!tc::worth<true>(p, code.W, &ts, 0)) {
+  if (!tc::worth<true>(p, code.W, strict, &ts, 0)) {
     for (int64_t t = pair + threadIdx.x * pairs; t < gx * gy; t += tc::kThreads * pairs) {
       int64_t tm, tn;
       grouped_tile(t, gx, gy, &tm, &tn);
-      for (int h = 0; h < NH; ++h) mark_tile(p, (tm * 2 + rank) * BM, (tn * NH + h) * BN);
+      for (int h = 0; h < NH; ++h) {
+        const int64_t m0 = (tm * 2 + rank) * BM, n0 = (tn * NH + h) * BN;
+        mark_tile(p, m0, n0);
+        if (m0 < p.M && n0 < p.N) tc::count(&tc::Check::left, 1);
+      }
     }
     return;
   }
@@ -728,7 +732,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc::kThreads, 1)
     }
     __syncthreads();
     if (changed) {
-      const bool w = tc::worth<false>(p, code.W, &ts, turn++);
+      const bool w = tc::worth<false>(p, code.W, false, &ts, turn++);
       if (threadIdx.x == 0) worth = w;
       __syncthreads();
     }
@@ -737,6 +741,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc::kThreads, 1)
       if (threadIdx.x < tc::kProducers) tc_finish<NH>(p, ok, at[0], at[1], buf, &ts);
     } else if (threadIdx.x < NH) {
       mark_tile(p, at[0], at[1] + threadIdx.x * BN);
+      if (at[0] < p.M && at[1] + threadIdx.x * BN < p.N) tc::count(&tc::Check::left, 1);
     }
   }
   if (threadIdx.x == 0 && tc::cta_rank() == 0 && !tc::usable(&ts, pr)) tc::count(&tc::Check::lost, 1);
@@ -905,8 +910,8 @@ int sm_count() {
 }
 
 // The encoding of a product; L = 0 where the tensor-core tile does not apply.
-tc::Code tc_code(int64_t K, int64_t lda, int64_t ldb) {
-  if (K < tc::kMinK || K > tc::kMaxK || lda > tc::kMaxLd || ldb > tc::kMaxLd) return tc::Code{0, 0};
+tc::Code tc_code(int64_t M, int64_t K, int64_t lda, int64_t ldb) {
+  if (M > tc::kMaxM || K < tc::kMinK || K > tc::kMaxK || lda > tc::kMaxLd || ldb > tc::kMaxLd) return tc::Code{0, 0};
   return tc::code_for(K);
 }
 
@@ -1015,10 +1020,14 @@ cudaError_t launch_minplus_gemm(const GemmParams& p, bool ring, cudaStream_t s, 
 // Only a product whose modeled DPX schedule is kTcGain times the tensor cores' is tried: where the operands' values are
 // against it the look at a sample costs 4 us.  At the line (1.5 to 2): 700^3, 23 against 25 us, is left out; 1024^3, 23
 // against 43 (47 where the sample says no), is tried.  2048^3 takes 31 against 271, 4096^3 128 against 1946.
-constexpr double kTcGain = 1.8;
+// Where the tensor cores decide a part of the tiles, that pays off as far as the DPX launch gets shorter by it.  Below a
+// modeled gain of kTcStrict it fills a wave or two and hardly does (operands of two diagonal blocks took 64 us at 1024^3
+// and 150 at 1500^3, DPX alone 43 and 127): there the sample has to speak for the whole product (`strict`).  Above it
+// does (2048^3: 188 us, DPX alone 289), and a launch in vain costs at most an eighth.
+constexpr double kTcGain = 1.8, kTcStrict = 8;
 cudaError_t launch_minplus_product(const GemmParams& p, cudaStream_t s) {
   bool marked = false;
-  const tc::Code code = tc_code(p.K, p.lda, p.ldb);
+  const tc::Code code = tc_code(p.M, p.K, p.lda, p.ldb);
   const GemmShape shape = gemm_shape(p.M, p.N, p.K);
   if (code.L) {
     const int64_t pairs = sm_count() / 2, gy = (p.M + 2 * BM - 1) / (2 * BM), KT = (p.K + tc::kBK - 1) / tc::kBK;
@@ -1032,11 +1041,12 @@ cudaError_t launch_minplus_product(const GemmParams& p, cudaStream_t s) {
     }
     if (shape.clocks > kTcGain * (double)(best + 16000)) {
       const int64_t n = gx * gy < pairs ? gx * gy : pairs;
+      const bool strict = shape.clocks < kTcStrict * (double)(best + 16000);
       const cudaError_t e =
           nh == 1 ? launch_kernel<minplus_tc_kernel<1>>(dim3((unsigned)(2 * n)), tc::kThreads, tc::smem_bytes(1), 1,
-                                                        false, s, p, code, gx, gy)
+                                                        false, s, p, code, gx, gy, strict)
                   : launch_kernel<minplus_tc_kernel<2>>(dim3((unsigned)(2 * n)), tc::kThreads, tc::smem_bytes(2), 1,
-                                                        false, s, p, code, gx, gy);
+                                                        false, s, p, code, gx, gy, strict);
       if (e != cudaSuccess) return e;
       marked = true;
     }
@@ -1347,7 +1357,7 @@ extern "C" rd_status rd_minplus_gemm_batched(const rd_gemm_problem* problems, in
     b.min_out = q.min_out;
     b.tiles_m = (q.M + BM - 1) / BM;
     b.tiles_n = (q.N + BN - 1) / BN;
-    b.code = tc_code(q.K, q.lda, q.ldb);
+    b.code = tc_code(q.M, q.K, q.lda, q.ldb);
     bp.tile_start[bp.count + 1] = bp.tile_start[bp.count] + b.tiles_m * b.tiles_n;
     const int64_t tcs = b.code.L ? (q.M + 2 * BM - 1) / (2 * BM) * ((q.N + 2 * BN - 1) / (2 * BN)) : 0;
     bp.tc_start[bp.count + 1] = bp.tc_start[bp.count] + tcs;

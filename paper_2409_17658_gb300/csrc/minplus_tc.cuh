@@ -37,7 +37,9 @@ __host__ __device__ constexpr int stage_bytes(int nh) { return kBytesA + nh * kB
 __host__ __device__ constexpr int stages(int nh) { return nh == 2 ? 3 : 4; }
 __host__ __device__ constexpr int smem_bytes(int nh) { return 1024 + stages(nh) * stage_bytes(nh); }
 constexpr int kMostFix = 64;                                          // undecided outputs of 128 x 256 computed term by term
+constexpr int64_t kMaxM = (int64_t)65535 * kBM;                       // as the DPX launch
 constexpr int64_t kMaxLd = 1 << 23;                                   // strides whose steps fit 32 bits
+constexpr int kLookStages = 40;                                       // tiles of fewer stages have no early look
 constexpr int64_t kMinK = 64, kMaxK = (int64_t)1 << 19;
 constexpr uint32_t kWaitRounds = 1u << 18;                            // bound of every mbarrier wait
 
@@ -47,7 +49,7 @@ struct Check {
   uint32_t wait_rounds;  // bound of the waits of a tile (those before the shared memory is given up keep kWaitRounds)
   int32_t hold_at;       // the first pair's MMA warp pauses before this stage, counted from 0 over its tiles (-1: never)
   uint32_t hold_us;      // for so many microseconds, as a warp that is kept from running would
-  uint32_t deaf;         // bit r: CTA r of a pair finds nothing in its half of the sample, whatever it holds
+  uint32_t deaf;         // bit r: CTA r of a pair finds nothing in its half of a sample, whatever it holds
   uint32_t decided, fixed, left, lost;  // parts of C written, outputs computed term by term, parts left to the DPX
                                         // launch, pairs of CTAs that lost their pipeline
 };
@@ -89,7 +91,7 @@ struct Shared {
   uint32_t bad;       // an operand outside the documented range in either CTA
   uint32_t lost[2];   // a wait ran out in either CTA, in an even or an odd phase of `all`; stays set
   uint32_t look[2];   // the early look: undecided outputs and outputs looked at, both CTAs
-  uint32_t vote[3][2];  // the sample's counts over both CTAs, one slot per question in turn
+  uint32_t vote[2][16];  // a sample's counts by group, from both CTAs; one slot per question in turn
   uint32_t cnt[2];    // undecided outputs of each 128 x 256 part
   uint32_t list[2][kMostFix];
 };
@@ -156,7 +158,7 @@ __device__ __forceinline__ void arrive_at(uint32_t bar) {
 // the other CTA has started and its barriers are ready), later the accumulator's TMEM columns.
 template <int NH>
 __device__ __forceinline__ void open(Shared* s) {
-  if (threadIdx.x == 0) {
+  if (threadIdx.x == kProducers) {  // not a thread that the first sample waits for
 #pragma unroll
     for (int i = 0; i < stages(NH); ++i) {
       mbar_init(&s->full[i], 2 * kProducers / 32);
@@ -164,7 +166,6 @@ __device__ __forceinline__ void open(Shared* s) {
     }
     mbar_init(&s->all, 1);
     s->lost[0] = s->lost[1] = 0;
-    s->vote[0][0] = s->vote[0][1] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   cluster_arrive();
@@ -250,42 +251,73 @@ __device__ __forceinline__ uint4 row8(const int16_t* row, int64_t e0, int64_t le
   return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-// Whether a product is worth trying: 256 vectors of 8 entries of each operand, spread over it, give the shares pa,
-// pb of entries below W; with K pa pb / 2 pairs expected to sum to at most W an output stays undecided with
-// probability exp(-K pa pb / 2), and a part of 32768 outputs needs nearly all of them decided.  Only speed hangs on
-// this, as long as both CTAs of a pair get the same answer: each reads half of the sample and adds what it finds to the
-// counts of both, so the answer is the same whatever the loads return.  All threads of the pair call it, for the
-// turn-th time; one load of each operand per thread, so it costs one memory latency.  FIRST: right behind open().
+// Whether a product is worth trying.  A sample of it: 16 groups of one row, 16 columns and 64 terms, spread over its
+// rows, columns and terms, 8 from each CTA.  It gives the pairs of entries that are `hits` (both below W, their sum at
+// most W), by group, and how many of the 256 outputs have none.  An output stays undecided with probability exp(-hits
+// among its K pairs), and a part of 32768 outputs needs nearly all of them decided: 32768 exp(-6.2) = 66.  So a product
+// is left to the DPX kernel
+//  * where K times the share of hits is below 6.2; if its tiles have an early look, only where it is so by more than the
+//    sample's deviation;
+//  * if `strict`, where clearly more outputs lack a hit than if the hits were spread evenly, or a quarter lacks one and
+//    the groups' hits differ by more than chance: rows, columns or blocks without a small entry, whose outputs stay
+//    undecided.
+// (The shares of small entries in A and in B alone, asked for before, passed operands in blocks, triangles or stripes of
+// 1024 to 2048 rows, which then took 1.1 to 1.55 times the DPX product's time.)
+// Only speed hangs on this, as long as both CTAs of a pair get the same answer: each writes what it finds to both, so the
+// answer is the same whatever the loads return.  All threads of the pair call it, for the turn-th time; the loads are in
+// flight together, so it costs one memory latency.  FIRST: right behind open().
 template <bool FIRST>
-__device__ __forceinline__ bool worth(const GemmParams& p, uint32_t W, Shared* s, uint32_t turn) {
-  const int tid = threadIdx.x;
-  const uint4 none = make_uint4(kInf2, kInf2, kInf2, kInf2);
-  uint4 va = none, vb = none;
-  if (tid < 128) {
-    const int i = tid + 128 * (int)cta_rank(), spread = (i & 15) * 16 + (i >> 4);
-    const int64_t ra = (i * p.M) >> 8, ca = ((spread * p.K) >> 8) & ~(int64_t)7;
-    const int64_t rb = (i * p.K) >> 8, cb = ((spread * p.N) >> 8) & ~(int64_t)7;
-    if (ca + 8 <= p.K) va = __ldg(reinterpret_cast<const uint4*>(p.A + ra * p.lda + ca));
-    if (cb + 8 <= p.N) vb = __ldg(reinterpret_cast<const uint4*>(p.B + rb * p.ldb + cb));
+__device__ __forceinline__ bool worth(const GemmParams& p, uint32_t W, bool strict, Shared* s, uint32_t turn) {
+  constexpr int kGroups = 16, kOutputs = 16 * kGroups, kTerms = 64;
+  constexpr uint32_t top = 0x80008000u;
+  const uint32_t tid = threadIdx.x, lane = tid & 31;
+  const uint32_t i = (tid >> 5) * 2 + cta_rank();  // the group; its row's place is another one
+  uint32_t* vote = s->vote[turn & 1];              // last read before the barrier of the question in between
+  const float need = __fdividef(6.2f * (kOutputs * kTerms), (float)p.K);
+  uint32_t hits = 0, any = 0;
+  if (tid < 16 * kGroups && p.N >= 8) {
+    // 32 bits hold these: K <= kMaxK, N <= ldb <= kMaxLd, M <= kMaxM
+    const uint32_t K = (uint32_t)p.K, last = (uint32_t)(p.N - 8) & ~7u;
+    const uint32_t M = (uint32_t)p.M;
+    // the last summand: offsets without a period, not one residue of the rows only
+    const uint32_t row = (((i * 5 + 3) & 15) * M >> 4) + (uint32_t)(0x904d2b2ff239863aull >> 4 * i & (M >= 256 ? 15 : 0));
+    uint32_t k = (((lane >> 1) * 16 + i) * K >> 8) & ~3u, col = ((i * (uint32_t)p.N >> 4) & ~7u) + (lane & 1) * 8;
+    if (k + 4 > K) k = (K - 4) & ~3u;
+    if (col > last) col = last;
+    const int16_t* b0 = p.B + (int64_t)k * p.ldb + col;
+    uint4 bv[4];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) bv[t] = __ldg(reinterpret_cast<const uint4*>(b0 + t * p.ldb));
+    const uint2 av = __ldg(reinterpret_cast<const uint2*>(p.A + (int64_t)row * p.lda + k));
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      const uint32_t a = ((t & 2) ? av.y : av.x) >> (16 * (t & 1)) & 0xFFFFu, b[4] = {bv[t].x, bv[t].y, bv[t].z, bv[t].w};
+      // a hit: an entry of B below this.  Entries are below 2^15, so bit 15 of a half of (b | top) - c says b >= c.
+      const uint32_t room = (a == 0 ? W : a < W ? W - a + 1 : 0) * 0x00010001u;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const uint32_t hit = ~((b[q] | top) - room) & top;
+        hits += __popc(hit);
+        any |= hit >> q;
+      }
+    }
+    hits = __reduce_add_sync(0xFFFFFFFFu, hits);
+    any = __reduce_or_sync(0xFFFFFFFFu, (lane & 1) ? any >> 4 : any);  // 8 of the 16 columns in each half's upper byte
+    if (deaf(cta_rank())) hits = 0, any = ~0u;
   }
-  const uint32_t w2 = W * 0x00010001u;
-  auto below = [&](const uint4& v) {
-    return (__popc(__vcmpltu2(v.x, w2)) + __popc(__vcmpltu2(v.y, w2)) + __popc(__vcmpltu2(v.z, w2)) +
-            __popc(__vcmpltu2(v.w, w2))) >> 4;
-  };
-  const int na = __reduce_add_sync(0xFFFFFFFFu, below(va));
-  const int nb = __reduce_add_sync(0xFFFFFFFFu, below(vb));
-  const uint32_t slot = turn % 3;
-  uint32_t* next = s->vote[(turn + 1) % 3];  // last read two questions ago, before the barrier of the one in between
-  if (tid == 0) next[0] = next[1] = 0;
   if (FIRST) cluster_wait();
-  if (tid < 128 && (tid & 31) < 2 && !deaf(cta_rank())) {
-    add_at(at_rank(&s->vote[slot][0], tid & 1), (uint32_t)na);
-    add_at(at_rank(&s->vote[slot][1], tid & 1), (uint32_t)nb);
-  }
+  if (tid < 16 * kGroups && lane < 2)
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(at_rank(&vote[i], lane)),
+                 "r"(hits | (16 - __popc(any & 0xFF00FF00u)) << 16)
+                 : "memory");
   cluster_sync();
-  const float pa = (float)s->vote[slot][0] * (1.f / 2048.f), pb = (float)s->vote[slot][1] * (1.f / 2048.f);
-  return (float)p.K * pa * pb * 0.5f >= 6.2f;  // 32768 exp(-6.2) = 66 undecided outputs
+  const uint32_t v = lane < kGroups ? vote[lane] : 0, mine = v & 0xFFFFu;
+  const uint32_t sum = __reduce_add_sync(0xFFFFFFFFu, v), squares = __reduce_add_sync(0xFFFFFFFFu, mine * mine);
+  const float found = (float)(sum & 0xFFFFu), none = (float)(sum >> 16), mean = found / kGroups;
+  const bool looks = p.K > (kLookStages - 1) * kBK;
+  if (!strict) return found >= need || (looks && (need - found) * (need - found) <= found);
+  return found >= need && none <= kOutputs * (__expf(-found / kOutputs) + 0.12f) &&
+         (none <= 0.25f * kOutputs || (float)squares <= kGroups * mean * (1.3f * mean + 2.f));
 }
 
 // One output by its terms, by a whole warp (operands inside [0, RD_INF]: no tile with other entries gets here).
@@ -410,7 +442,7 @@ __device__ __forceinline__ bool tile(const GemmParams& p, const int64_t m0, cons
   const int KT = (int)((p.K + kBK - 1) / kBK);
   // The early look (an eighth of the way) costs 2 us a tile, 8 % of a product at K = 1024; a tile of fewer stages than
   // this that turns out hopeless costs at most 20.
-  const int check = KT >= 40 ? KT >> 3 : -1;
+  const int check = KT >= kLookStages ? KT >> 3 : -1;
 
   if (tid == 0) s->at[0] = m0, s->at[1] = n0;
   if (tid == 0) s->bad = s->look[0] = s->look[1] = s->cnt[0] = s->cnt[1] = 0;

@@ -151,3 +151,63 @@ def test_operands_and_result_in_interleaved_rows(rd, orc, M, N, K):
     assert_product(orc, a, b, C)
     C[:, :N] = -7
     assert torch.equal(parent, before)
+
+
+def structured(kind, n, seed):
+    """Operands uniform in [0, 32] with infinity at probability 1/2, and infinite by a pattern."""
+    a, b = draw(n, n, 33, 0.5, seed), draw(n, n, 33, 0.5, seed + 1)
+    if kind == "blocks":  # two diagonal blocks
+        for x in (a, b):
+            x[: n // 2, n // 2:] = x[n // 2:, : n // 2] = INF
+    elif kind == "triangle":
+        for x in (a, b):
+            x[np.tril_indices(n, -1)] = INF
+    elif kind == "columns":
+        b[:, ::2] = INF
+    elif kind == "odd rows":
+        a[1::2] = INF
+    elif kind == "half the rows":
+        a[: n // 2] = INF
+    elif kind == "apart":  # small entries of A meet large ones of B
+        a[:, : n // 2] = np.where(a[:, : n // 2] == INF, INF, a[:, : n // 2] + 0x800)
+        b[n // 2:] = np.where(b[n // 2:] == INF, INF, b[n // 2:] + 0x800)
+    return a, b
+
+
+@pytest.mark.parametrize("n", [1024, 1500])
+@pytest.mark.parametrize("kind", ["even", "blocks", "triangle", "columns", "odd rows", "half the rows", "apart"])
+def test_the_sample_sees_what_stays_undecided(rd, orc, kind, n):
+    """Sizes where the DPX launch gains nothing from the tiles that the tensor cores decide: none is tried unless the
+    hits are spread over the whole product."""
+    a, b = structured(kind, n, 11)
+    C = result(n, n)
+    rd.minplus_gemm(upload(a), upload(b), C, n, n, n)
+    seen = check(rd)
+    want = (parts(n, n), 0) if kind == "even" else (0, parts(n, n))
+    assert (seen["decided"], seen["left"]) == want, seen
+    assert_product(orc, a, b, C)
+
+
+def test_large_products_are_decided_in_part(rd, orc):
+    """2048^3 with the upper half of A's rows infinite: the lower half's parts on the tensor cores, the others not."""
+    n = 2048
+    a, b = structured("half the rows", n, 21)
+    C = result(n, n)
+    rd.minplus_gemm(upload(a), upload(b), C, n, n, n)
+    seen = check(rd)
+    assert (seen["decided"], seen["left"]) == (parts(n, n) // 2, parts(n, n) // 2), seen
+    assert_product(orc, a, b, C)
+
+
+def test_outputs_computed_term_by_term(rd, orc):
+    """A few rows' worth of single outputs without a small pair: computed beside the decided ones, not left."""
+    n = 1100
+    a, b = draw(n, n, 33, 0.5, 31), draw(n, n, 33, 0.5, 32)
+    a[700] = np.where(np.arange(n) % 64 == 0, a[700], INF)  # 17 terms: part of the row stays undecided
+    b[:, 40:1000] = np.where(b[:, 40:1000] == INF, INF, b[:, 40:1000] % 4)
+    b[:, :8] = np.where(np.arange(n)[:, None] % 60 == 0, b[:, :8], INF)
+    C = result(n, n)
+    rd.minplus_gemm(upload(a), upload(b), C, n, n, n)
+    seen = check(rd)
+    assert seen["decided"] + seen["left"] == parts(n, n) and seen["decided"] > 0, seen
+    assert_product(orc, a, b, C)
