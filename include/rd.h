@@ -187,7 +187,8 @@ rd_status rd_minplus_gemv(const int16_t *x, const int16_t *B, int64_t ldb, int16
  * rd_minplus_gemm_batched -- `count` (<= 128) independent products
  * C_i = A_i (x) B_i, each with the conventions of rd_minplus_gemm (min_out may
  * be null), in one persistent launch over the tensor cores (one CTA per SM, in
- * pairs) and one over the DPX units for the tiles that those leave (two per SM):
+ * pairs; not where the batch is too small for it to pay) and one over the DPX
+ * units for the tiles that those leave (two per SM):
  * each walks the concatenated tile list of all products, longest tiles (largest
  * K) first, so small products run side by side and the tail of a large one is
  * filled by others.  The problem table travels in the kernel's parameters (no

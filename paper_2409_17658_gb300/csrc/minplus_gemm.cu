@@ -26,6 +26,7 @@
 //    whose terms all involve RD_INF ends exactly at RD_INF.
 #include <cooperative_groups.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "minplus_tc.cuh"
@@ -702,7 +703,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc::kThreads, 1)
   if (threadIdx.x == 0) cur = -1;
   tc::open<NH>(&ts);
   tc::cluster_wait();
-  tc::take_accumulator<NH>(&ts);
+  bool taken = false;  // the accumulator's columns, from the first tile on that is tried
   tc::Progress pr;
   uint32_t turn = 0;
 #pragma unroll 1
@@ -737,6 +738,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc::kThreads, 1)
       __syncthreads();
     }
     if (worth) {
+      if (!taken) tc::take_accumulator<NH>(&ts);
+      taken = true;
       const bool ok = tc::usable(&ts, pr) && tc::tile<NH>(p, at[0], at[1], code, buf, &ts, pr);
       if (threadIdx.x < tc::kProducers) tc_finish<NH>(p, ok, at[0], at[1], buf, &ts);
     } else if (threadIdx.x < NH) {
@@ -744,6 +747,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc::kThreads, 1)
       if (at[0] < p.M && at[1] + threadIdx.x * BN < p.N) tc::count(&tc::Check::left, 1);
     }
   }
+  if (!taken) return;
   if (threadIdx.x == 0 && tc::cta_rank() == 0 && !tc::usable(&ts, pr)) tc::count(&tc::Check::lost, 1);
   tc::close<NH>(&ts);
 }
@@ -1370,7 +1374,25 @@ extern "C" rd_status rd_minplus_gemm_batched(const rd_gemm_problem* problems, in
   const int sms = sm_count();
   const int64_t total = bp.tile_start[bp.count];
   const int64_t grid = total < 2 * (int64_t)sms ? total : 2 * (int64_t)sms;  // two resident CTAs per SM
-  const int64_t tcs = bp.tc_start[bp.count], pairs = tcs < sms / 2 ? tcs : sms / 2;
+  // The tensor cores are tried where the batch passes the line that single products have, modeled alike: the tiles'
+  // clocks over all SMs (pairs), at least those of the longest tile.  Below it a batch pays the launch and the samples
+  // for nothing: 128 products of 64^3 16 -> 37 us, 64 of 100^3 28 -> 53 (uniform [0, 32]), before this line.  Above it a
+  // batch against which the samples are pays 5 to 10 us: 16 of 500^3, entries over the whole range, 96 -> 100 (31 us
+  // where they are for it).
+  double dpx_all = 0, dpx_most = 0, tc_all = 0, tc_most = 0;
+  for (int i = 0; i < bp.count; ++i) {
+    const double kt = (double)((bp.p[i].K + BK - 1) / BK) * BN * BK, KT = (double)((bp.p[i].K + tc::kBK - 1) / tc::kBK);
+    const double one = kt / 0.88 + 6000, two = 1540 * KT + 14000;
+    dpx_all += (double)(bp.tile_start[i + 1] - bp.tile_start[i]) * (kt / 0.93 + 3000) / sms;
+    if (one > dpx_most) dpx_most = one;
+    if (!bp.p[i].code.L) continue;
+    tc_all += (double)(bp.tc_start[i + 1] - bp.tc_start[i]) * two / (sms / 2);
+    if (two > tc_most) tc_most = two;
+  }
+  const bool worth = std::max(dpx_all, dpx_most) > kTcGain * (std::max(tc_all, tc_most) + 16000);
+  if (!worth)  // no tile is marked
+    for (int i = 0; i < bp.count; ++i) bp.p[i].code = tc::Code{0, 0};
+  const int64_t tcs = worth ? bp.tc_start[bp.count] : 0, pairs = tcs < sms / 2 ? tcs : sms / 2;
   if (pairs > 0)
     e = launch_kernel<minplus_tc_batched_kernel<2>>(dim3((unsigned)(2 * pairs)), tc::kThreads, tc::smem_bytes(2), 1, false, s,
                                                     bp);

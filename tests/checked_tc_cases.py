@@ -211,3 +211,19 @@ def test_outputs_computed_term_by_term(rd, orc):
     seen = check(rd)
     assert seen["decided"] + seen["left"] == parts(n, n) and seen["decided"] > 0, seen
     assert_product(orc, a, b, C)
+
+
+@pytest.mark.parametrize("count,n,tried", [(1, 100, False), (64, 100, False), (128, 64, False), (100, 128, False),
+                                           (1, 200, True), (16, 500, True), (128, 256, True)])
+def test_small_batches_stay_on_dpx(rd, orc, count, n, tried):
+    """The tensor cores are tried where the modeled schedules say so, for the batch as a whole."""
+    host = [(draw(n, n, 4, 0.1, 40 + i), draw(n, n, 4, 0.1, 90 + i)) for i in range(3)]
+    dev = [(upload(a), upload(b)) for a, b in host]
+    outs = [result(n, n) for _ in range(count)]
+    rd.minplus_gemm_batched([(*dev[i % 3], C, n, n, n, None) for i, C in enumerate(outs)])
+    seen = check(rd)
+    assert (seen["decided"], seen["left"]) == (count * parts(n, n) if tried else 0, 0), seen
+    want = [orc.minplus_i16(a, b) for a, b in host]
+    for i, C in enumerate(outs):
+        got = C.cpu().numpy()
+        assert np.array_equal(got[:, :n].astype(np.int32), want[i % 3]) and (got[:, n:] == -7).all()
