@@ -154,11 +154,21 @@ __global__ void __launch_bounds__(128) sparse_minplus_kernel(SparseArgs a) {
 // The same product for small operands: one warp = one block of R rows x 256 columns, a CTA's warps neighbouring blocks
 // over the same columns, their records staged by each warp for itself.  Finer pieces than the 2048 columns of the CTA
 // above, no barrier between a block's chunks, and neighbours read mostly the same rows of B (words that differ in
-// their last letters), which they find in the SM's L1 cache.  Per product at R = 2: m = 5 19.2 -> 12.7 us, m = 6 35 ->
-// 19, m = 7 92 -> 58; at m = 8 (7411 rows) it loses, 455 against 502 us, m = 9 4.75 against 6.5 ms: the blocks of one
-// CTA differ in length, and their rows no longer fit L1.
+// their last letters), which they find in the SM's L1 cache.  Per product with A(G) at R = 2: m = 5 18.6 -> 14.4 us, m = 6
+// 35 -> 22.8, m = 7 92 -> 67; at m = 8 (7411 rows) it loses, 455 against 502 us, m = 9 4.75 against 5.9 ms: the blocks of
+// one CTA differ in length, and their rows no longer fit L1.
 constexpr int kRowsSlab = 256, kMostWarps = 16;
 constexpr int64_t kRowsMost = 4096;  // rows and columns
+// Within that, it is taken where the CTA above wastes its lanes (the last 2048-column slab mostly empty: at most 0.65 of
+// all slabs' columns exist) or there are few of them (at most 3.5 per SM), and at R = 8, whose CTAs are the longest.
+// Elsewhere random operands, which share no rows of B, lose: 4000^3 at 2 % of the entries, R = 2, 148 against 204 us;
+// 1500 x 2000 x 1900 at 3 % 35 against 44.  On this side: 1500 x 2000 x 1200 33 -> 27, 500 x 2000 x 4000 33 -> 27, the
+// same with R = 8 135 -> 76.
+bool rows_suit(int R, int64_t M, int64_t N, int sms) {
+  if (M > kRowsMost || N > kRowsMost) return false;
+  const int64_t slabs = (N + 2047) / 2048, blocks = (M + R - 1) / R;
+  return R == 8 || 20 * N <= 13 * 2048 * slabs || 2 * blocks * slabs <= 7 * (int64_t)sms;
+}
 
 template <int R, bool RING>
 __global__ void __launch_bounds__(32 * kMostWarps) sparse_rows_kernel(SparseArgs a) {
@@ -288,12 +298,10 @@ cudaError_t launch_sparse_tma(int R, const SparseArgs& a, int32_t* err, cudaStre
 }
 
 template <bool RING>
-cudaError_t launch_sparse_rows(int R, const SparseArgs& a, cudaStream_t s) {
+cudaError_t launch_sparse_rows(int R, const SparseArgs& a, int sms, cudaStream_t s) {
   const int64_t nb = (a.M + R - 1) / R;
   const int64_t gy = (a.Ncols + kRowsSlab - 1) / kRowsSlab;
   // as many neighbouring blocks per CTA as leave every SM one and a half CTAs
-  int dev = 0, sms = 148;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   int warps = kMostWarps;
   while (warps > 1 && 2 * ((nb + warps - 1) / warps * gy) < 3 * (int64_t)sms) warps /= 2;
   const dim3 grid((unsigned)((nb + warps - 1) / warps), (unsigned)gy);
@@ -317,7 +325,9 @@ cudaError_t launch_sparse(int R, const SparseArgs& a, cudaStream_t s) {
   const int threads = 128;
   const int64_t gy = (a.Ncols + threads * 16 - 1) / (threads * 16);
   if (nb <= 0 || gy <= 0) return cudaSuccess;
-  if (a.M <= kRowsMost && a.Ncols <= kRowsMost) return launch_sparse_rows<RING>(R, a, s);
+  int dev = 0, sms = 148;
+  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (rows_suit(R, a.M, a.Ncols, sms)) return launch_sparse_rows<RING>(R, a, sms, s);
   if (nb > 0x7FFFFFFF || gy > 65535) return cudaErrorInvalidConfiguration;
   const dim3 grid((unsigned)nb, (unsigned)gy);
   switch (R) {
