@@ -717,6 +717,12 @@ rd_status rd_tune_lookup(int mode, int key, int aux, rd_tune_entry_t *out);
  * that suits the product and would not exceed four waves of CTAs (one
  * warm-up, then reps >= 1 timed products), records the fastest in the table
  * (replacing an entry with the same key) and returns it in *best (nullable).
+ * The shape that the product runs without an entry is timed too, if it is not
+ * one of these (S = 3, 5, 6 or 7, or beyond the waves): where it is the fastest
+ * and the table cannot hold it, the table is left without an entry for the key
+ * (rd_tune_lookup: RD_NOT_FOUND), and *best is the fastest of the others.
+ * Times and entries are of the DPX launch: a product that is tried on the tensor
+ * cores takes the shape for the tiles that they leave, and ms is not its time.
  * Synchronous.
  */
 rd_status rd_tune_gemm(const int16_t *A, int64_t lda, const int16_t *B, int64_t ldb, int16_t *C, int64_t ldc,

@@ -981,7 +981,8 @@ cudaError_t launch_minplus_gemm(const GemmParams& p, bool ring, cudaStream_t s, 
   int S = 1;     // ring mode and the diagonal output keep one CTA per tile (no diagonal in the split form)
   int tile = 0;  // 0: BM x BN, 1: BM x BN_NARROW (no ring mode, no diagonal)
   if (force_splitk > 0) {
-    if (ring || p.diag_out != nullptr || !splitk_suits(force_splitk, p.K) || force_tile < 0 || force_tile > 1)
+    if (ring || p.diag_out != nullptr || force_splitk > 8 || !slices_full(force_splitk, p.K) || force_tile < 0 ||
+        force_tile > 1)
       return cudaErrorInvalidValue;
     S = force_splitk;
     tile = force_tile;

@@ -96,18 +96,20 @@ struct GemmShape {
 };
 
 // Launchers implemented in the .cu files.
-// force_splitk > 0 (not in ring mode): split K by exactly that factor, with tile shape force_tile (0: 128 x
+// force_splitk > 0 (not in ring mode): split K by exactly that factor (1..8), with tile shape force_tile (0: 128 x
 // 256, 1: 128 x 128) -- the autotuner's trials; else the tuning table's factor and tile for the product's
 // size class, else the modeled shape (`shape`, where the caller has it).  marked: only the tiles that the tensor-core
 // launch before it has marked.
 cudaError_t launch_minplus_gemm(const GemmParams& p, bool ring, cudaStream_t s, int force_splitk = 0,
                                 int force_tile = 0, bool marked = false, const GemmShape* shape = nullptr);
 bool splitk_suits(int S, int64_t K);         // S in {1, 2, 4, 8} and every K slice non-empty
+GemmShape gemm_shape(int64_t M, int64_t N, int64_t K);  // the modeled shape (S in 1..8)
 int64_t gemm_tiles(int64_t M, int64_t N);  // output tiles (CTAs of an unsplit launch)
 
-// The tuning table (tune.cu): lookup and insert-or-replace by (mode, key, aux).
+// The tuning table (tune.cu): lookup, insert-or-replace and removal by (mode, key, aux).
 bool tune_find(int mode, int key, int aux, rd_tune_entry_t* out);
 bool tune_put(const rd_tune_entry_t& e);
+void tune_drop(const rd_tune_entry_t& e);
 
 // Row-split passes (split.cu): whether slab width W fits with max_slots staged rows.
 bool split_width_fits(int W, int max_slots);

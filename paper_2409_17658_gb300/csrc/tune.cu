@@ -108,6 +108,16 @@ bool tune_put(const rd_tune_entry_t& e) {
   return true;
 }
 
+void tune_drop(const rd_tune_entry_t& e) {
+  Table& t = table();
+  std::lock_guard<std::mutex> g(t.mu);
+  for (int i = 0; i < t.n; ++i)
+    if (same_key(t.e[i], e)) {
+      t.e[i] = t.e[--t.n];
+      return;
+    }
+}
+
 }  // namespace rd
 
 using namespace rd;
@@ -176,6 +186,22 @@ extern "C" rd_status rd_tune_gemm(const int16_t* A, int64_t lda, const int16_t* 
   t.key = rd_tune_bucket(M > N ? M : N);
   t.aux = rd_tune_bucket(K);
   t.ms = -1.f;
+  rd_status rc = RD_OK;
+  auto time_shape = [&](int S, int tile) {
+    return time_calls(
+        [&]() -> rd_status {
+          const cudaError_t e = launch_minplus_gemm(p, false, s, S, tile);
+          if (e != cudaSuccess) {
+            set_cuda_error(e);
+            return RD_ERR_CUDA;
+          }
+          return RD_OK;
+        },
+        reps, ev.e0, ev.e1, s, &rc);
+  };
+  // the shape that a product without an entry runs, which may be one that the loop below does not time
+  const GemmShape own = gemm_shape(M, N, K);
+  bool own_timed = false;
   const int cands[4] = {1, 2, 4, 8};
   for (int tile = 0; tile < 2; ++tile) {
     // the wide tile runs 2 CTAs per SM, the narrow one 3
@@ -183,18 +209,9 @@ extern "C" rd_status rd_tune_gemm(const int16_t* A, int64_t lda, const int16_t* 
     for (int S : cands) {
       if (!splitk_suits(S, K) || (S > 1 && tiles * S > 4 * wave)) continue;
       if (tile && tiles > 4 * wave) continue;  // the narrow tile only for products of a few waves
-      rd_status rc = RD_OK;
-      const float ms = time_calls(
-          [&]() -> rd_status {
-            const cudaError_t e = launch_minplus_gemm(p, false, s, S, tile);
-            if (e != cudaSuccess) {
-              set_cuda_error(e);
-              return RD_ERR_CUDA;
-            }
-            return RD_OK;
-          },
-          reps, ev.e0, ev.e1, s, &rc);
+      const float ms = time_shape(S, tile);
       if (rc != RD_OK) return rc;
+      own_timed |= S == own.S && tile == own.tile;
       if (t.ms < 0.f || ms < t.ms) {
         t.p[0] = S;
         t.p[1] = tile;
@@ -202,7 +219,20 @@ extern "C" rd_status rd_tune_gemm(const int16_t* A, int64_t lda, const int16_t* 
       }
     }
   }
-  if (!tune_put(t)) return RD_ERR_NOMEM;  // the table is full
+  bool keep = true;
+  if (!own_timed) {
+    const float ms = time_shape(own.S, own.tile);
+    if (rc != RD_OK) return rc;
+    if (ms <= t.ms && is_pow2_le8(own.S)) {
+      t.p[0] = own.S;
+      t.p[1] = own.tile;
+      t.ms = ms;
+    } else if (ms <= t.ms) {  // no entry says it, and none is needed
+      keep = false;
+      tune_drop(t);
+    }
+  }
+  if (keep && !tune_put(t)) return RD_ERR_NOMEM;  // the table is full
   if (best) *best = t;
   return RD_OK;
 }
