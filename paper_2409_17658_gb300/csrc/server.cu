@@ -148,7 +148,11 @@ rd_status admit_split(rd_server* sv, Job* j, size_t base) {
     free_job(sv, j);
     return (j->need > sv->budget) ? RD_ERR_ARG : RD_ERR_NOMEM;
   }
-  if (cudaMalloc(&j->plan, pbytes) != cudaSuccess) return RD_ERR_CUDA;
+  cudaError_t e = cudaMalloc(&j->plan, pbytes);
+  if (e != cudaSuccess) {
+    rd::set_cuda_error(e);
+    return RD_ERR_CUDA;
+  }
   j->footprint += pbytes;
   sv->used += pbytes;
   rc = rd_split_plan(j->m, sj, j->plan, pbytes, &j->split.info, sv->stream);
@@ -159,7 +163,11 @@ rd_status admit_split(rd_server* sv, Job* j, size_t base) {
     free_job(sv, j);
     return (j->need > sv->budget) ? RD_ERR_ARG : RD_ERR_NOMEM;
   }
-  if (cudaMalloc(&j->X, xbytes) != cudaSuccess) return RD_ERR_CUDA;
+  e = cudaMalloc(&j->X, xbytes);
+  if (e != cudaSuccess) {
+    rd::set_cuda_error(e);
+    return RD_ERR_CUDA;
+  }
   j->footprint += xbytes;
   sv->used += xbytes;
   j->split.plan = j->plan;
@@ -189,6 +197,7 @@ rd_status admit(rd_server* sv, Job* j) {
   j->footprint = base;
   sv->used += base;
   rd_status rc = (e == cudaSuccess) ? RD_OK : RD_ERR_CUDA;
+  if (e != cudaSuccess) rd::set_cuda_error(e);
   if (rc == RD_OK) rc = rd_build_transfer(j->m, j->A, j->ld, sv->stream);
   if (use_split && rc == RD_OK) {
     rc = admit_split(sv, j, base);
@@ -209,8 +218,10 @@ rd_status admit(rd_server* sv, Job* j) {
   }
   if (!use_split && rc == RD_OK) {
     e = cudaMalloc(&j->rec, rec_bytes);
-    if (e != cudaSuccess) rc = RD_ERR_CUDA;
-    else {
+    if (e != cudaSuccess) {
+      rd::set_cuda_error(e);
+      rc = RD_ERR_CUDA;
+    } else {
       j->footprint += rec_bytes;
       sv->used += rec_bytes;
     }

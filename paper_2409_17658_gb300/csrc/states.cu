@@ -237,7 +237,10 @@ int build_rows_per_cta(int64_t n, int64_t ctiles) {
 
 }  // namespace
 
-void set_cuda_error(cudaError_t e) { g_last_error = cudaGetErrorString(e); }
+void set_cuda_error(cudaError_t e) {
+  g_last_error = cudaGetErrorString(e);
+  cudaGetLastError();  // reported here: a later call's check of its own launch must not find it
+}
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 }  // namespace rd
