@@ -783,7 +783,9 @@ rd_status rd_measure_addmin_peak(void *work_dev, size_t work_bytes, int64_t trip
  * search: in one CTA (rd_power_until_periodic) when C_m <= 128 (m <= 4), else
  * by rd_power_until_periodic_split, on the current device, in device memory this
  * call allocates and frees (about 7.3 powers of C_m x C_m int16: 7 GB at m = 9,
- * 61 GB at m = 10; RD_ERR_NOMEM when that does not fit); the result (gamma for
+ * 61 GB at m = 10; where that does not fit, from m = 9 on, 3 powers and a column
+ * chunk of the intermediate: 3.4 GB, 28 GB and 225 GB at m = 9, 10 and 11;
+ * RD_ERR_NOMEM when that does not fit either); the result (gamma for
  * n < k + p, and (k, p, q)) is cached per m for the life of the process, and later calls evaluate the
  * solution of the finite-difference equation of Prop. 7 on the host:
  * gamma(n) = gamma(k + (n - k) mod p) + q floor((n - k) / p) for n >= k.

@@ -451,33 +451,51 @@ rd_status compute_cached(int m, Cached* out) {
   rd_padded_dim(N, &ld);
   const int split_j = rd_split_default_j(m);
   const size_t mat = (size_t)N * (size_t)ld * 2;
-  // Low-memory form when A(G), 8 ring slots and the whole intermediate of the row split do not fit (m >= 11:
-  // 73 GB per power): 3 ring slots with A(G) built in the first (it is read only for the first power), the
-  // intermediate in 8192-column chunks, and a repeat whose earlier power has left the ring verified by
-  // re-deriving that power (rd_power_until_periodic_split).
-  size_t free_b = 0, total_b = 0;
-  cudaMemGetInfo(&free_b, &total_b);
-  const bool lowmem = split_j > 0 && N > 8192 && mat * 11 > free_b;
-  // The row-split search keeps 6 slots and builds A(G) in the first of them too: the repeats of A(G) found so far are
-  // at most 5 powers apart for these sizes, and one that is not is verified by re-deriving, as above.  Allocating and
-  // freeing costs 0.7 ms per GB: with A(G) beside 8 slots (16 for N <= 8192) a first query took 42.8 ms at m = 9, now
-  // 40.4.
+  // The row-split search keeps 6 slots and builds A(G) in the first of them too (it is read only for the first power):
+  // the repeats of A(G) found so far are at most 5 powers apart, and one that is not is verified by re-deriving the
+  // earlier power (rd_power_until_periodic_split).  Allocating and freeing costs 0.7 ms per GB: with A(G) beside 8 slots
+  // (16 for N <= 8192) a first query took 42.8 ms at m = 9, now 40.4.
   const bool in_ring = split_j > 0 && N > kSmallN;
-  const int slots = lowmem ? 3 : in_ring ? 6 : (N <= 8192) ? 16 : 8;
-  size_t wbytes = 0;
-  rd_power_work_bytes(N, ld, kGammaKmax, slots, &wbytes);
-  int16_t* A = nullptr;
-  int16_t* A_own = nullptr;
-  void* work = nullptr;
-  cudaStream_t s = nullptr;
-  rd_status rc = RD_OK;
   std::vector<int64_t> g((size_t)kGammaKmax + 1);
   int32_t k = 0, p = 0;
   int64_t q = 0;
+  rd_status rc = RD_OK;
+  cudaStream_t s = nullptr;
+  void* plan = nullptr;
+  rd_split_info_t info{};
   cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
-  if (e == cudaSuccess && !in_ring) e = cudaMalloc(&A_own, mat);
-  if (e == cudaSuccess) e = cudaMalloc(&work, wbytes);
-  if (e != cudaSuccess) {
+  size_t free_b = 0, total_b = 0, least = 0;
+  cudaMemGetInfo(&free_b, &total_b);
+  rd_power_work_bytes(N, ld, kGammaKmax, 3, &least);
+  if (in_ring && least > total_b) {  // no form fits this device (m >= 12)
+    if (e == cudaSuccess) e = cudaErrorMemoryAllocation;
+  } else if (in_ring) {  // the plan first: it tells the size of the intermediate
+    size_t pbytes = 0;
+    rc = rd_split_plan_bytes(m, split_j, &pbytes);
+    if (rc == RD_OK && e == cudaSuccess) e = cudaMalloc(&plan, pbytes);
+    if (rc == RD_OK && e == cudaSuccess) rc = rd_split_plan(m, split_j, plan, pbytes, &info, s);
+  }
+  int slots = in_ring ? 6 : (N <= 8192) ? 16 : 8;
+  size_t wbytes = 0;
+  rd_power_work_bytes(N, ld, kGammaKmax, slots, &wbytes);
+  // Low-memory form when 6 slots and the whole intermediate do not fit beside each other (m >= 11: 73 GB per power): 3
+  // slots and the intermediate in 8192-column chunks.  The margin covers the rounding of the two allocations.
+  bool lowmem = false;
+  if (in_ring && N > 8192) {
+    cudaMemGetInfo(&free_b, &total_b);
+    lowmem = wbytes + (size_t)info.x_rows * (size_t)ld * 2 + ((size_t)64 << 20) > free_b;
+    if (lowmem) {
+      slots = 3;
+      rd_power_work_bytes(N, ld, kGammaKmax, slots, &wbytes);
+      info.chunk_cols = 8192;
+    }
+  }
+  int16_t* A = nullptr;
+  int16_t* A_own = nullptr;
+  void* work = nullptr;
+  if (rc == RD_OK && e == cudaSuccess && !in_ring) e = cudaMalloc(&A_own, mat);
+  if (rc == RD_OK && e == cudaSuccess) e = cudaMalloc(&work, wbytes);
+  if (rc == RD_OK && e != cudaSuccess) {
     set_cuda_error(e);
     rc = (e == cudaErrorMemoryAllocation) ? RD_ERR_NOMEM : RD_ERR_CUDA;
   }
@@ -497,19 +515,12 @@ rd_status compute_cached(int m, Cached* out) {
     if (s) cudaStreamDestroy(s);
     return finish_cached(rc, g, k, p, q, out);
   }
-  if (rc == RD_OK && split_j > 0) {
+  if (in_ring) {
     // the row-split step: A(G) (x) P_k from the row rules, in two passes
-    size_t pbytes = 0;
-    void* plan = nullptr;
     int16_t* X = nullptr;
-    rd_split_info_t info{};
-    rc = rd_split_plan_bytes(m, split_j, &pbytes);
-    if (rc == RD_OK) e = cudaMalloc(&plan, pbytes);
-    if (rc == RD_OK && e == cudaSuccess) rc = rd_split_plan(m, split_j, plan, pbytes, &info, s);
-    if (lowmem) info.chunk_cols = 8192;
     const int64_t ldx = lowmem ? info.chunk_cols : ld;
-    if (rc == RD_OK && e == cudaSuccess) e = cudaMalloc(&X, (size_t)info.x_rows * (size_t)ldx * 2);
-    if (e != cudaSuccess) {
+    if (rc == RD_OK) e = cudaMalloc(&X, (size_t)info.x_rows * (size_t)ldx * 2);
+    if (rc == RD_OK && e != cudaSuccess) {
       set_cuda_error(e);
       rc = (e == cudaErrorMemoryAllocation) ? RD_ERR_NOMEM : RD_ERR_CUDA;
     }
@@ -518,7 +529,6 @@ rd_status compute_cached(int m, Cached* out) {
     if (s) cudaStreamSynchronize(s);
     if (plan) cudaFree(plan);
     if (X) cudaFree(X);
-    if (A_own) cudaFree(A_own);
     if (work) cudaFree(work);
     if (s) cudaStreamDestroy(s);
     return finish_cached(rc, g, k, p, q, out);
