@@ -1409,9 +1409,9 @@ extern "C" rd_status rd_tc_check(const uint32_t* settings, uint32_t* counts) {
   tc::Check c;
   cudaError_t e = cudaMemcpyFromSymbol(&c, tc::g_check, sizeof(c));
   if (e == cudaSuccess) {
-    if (counts) counts[0] = c.decided, counts[1] = c.fixed, counts[2] = c.left, counts[3] = c.lost;
+    if (counts) counts[0] = c.decided, counts[1] = c.fixed, counts[2] = c.left, counts[3] = c.lost, counts[4] = c.early;
     if (settings) c.wait_rounds = settings[0], c.hold_at = (int32_t)settings[1], c.hold_us = settings[2], c.deaf = settings[3];
-    c.decided = c.fixed = c.left = c.lost = 0;
+    c.decided = c.fixed = c.left = c.lost = c.early = 0;
     e = cudaMemcpyToSymbol(tc::g_check, &c, sizeof(c));
   }
   if (e != cudaSuccess) { set_cuda_error(e); return RD_ERR_CUDA; }

@@ -50,11 +50,12 @@ struct Check {
   int32_t hold_at;       // the first pair's MMA warp pauses before this stage, counted from 0 over its tiles (-1: never)
   uint32_t hold_us;      // for so many microseconds, as a warp that is kept from running would
   uint32_t deaf;         // bit r: CTA r of a pair finds nothing in its half of a sample, whatever it holds
-  uint32_t decided, fixed, left, lost;  // parts of C written, outputs computed term by term, parts left to the DPX
-                                        // launch, pairs of CTAs that lost their pipeline
+  // parts of C written, outputs computed term by term, parts left to the DPX launch, pairs of CTAs that lost their
+  // pipeline, tiles left by the early look
+  uint32_t decided, fixed, left, lost, early;
 };
 #ifdef RD_CHECKED
-__device__ Check g_check = {kWaitRounds, -1, 0, 0, 0, 0, 0, 0};
+__device__ Check g_check = {kWaitRounds, -1, 0, 0, 0, 0, 0, 0, 0};
 __device__ __forceinline__ uint32_t wait_rounds() { return *(volatile uint32_t*)&g_check.wait_rounds; }
 __device__ __forceinline__ void count(uint32_t Check::*what, uint32_t n) { atomicAdd(&(g_check.*what), n); }
 __device__ __forceinline__ void hold(uint32_t stage) {
@@ -619,6 +620,7 @@ __device__ __forceinline__ bool tile(const GemmParams& p, const int64_t m0, cons
     if (stop == KT) break;
     if (look()) {
       if (lost_by(s, f.pr.all)) settle();
+      else if (tid == 0 && rank == 0) count(&Check::early, 1);
       pr = f.pr;
       return false;
     }

@@ -30,9 +30,9 @@ def rd():
 def check(rd, wait_rounds=1 << 18, hold_at=-1, hold_us=0, deaf=0):
     """Applies settings (by default: the ordinary ones); returns the counts since the last call."""
     settings = (ctypes.c_uint32 * 4)(wait_rounds, hold_at & 0xFFFFFFFF, hold_us, deaf)
-    counts = (ctypes.c_uint32 * 4)()
+    counts = (ctypes.c_uint32 * 5)()
     assert rd._lib().rd_tc_check(settings, counts) == rd.RD_OK
-    return dict(zip(("decided", "fixed", "left", "lost"), counts))
+    return dict(zip(("decided", "fixed", "left", "lost", "early"), counts))
 
 
 @pytest.fixture(autouse=True)
@@ -96,7 +96,7 @@ def test_a_wait_that_runs_out_leaves_the_rest_of_the_pair(rd, orc, M, N, K, stag
     C.fill_(-7)
     rd.minplus_gemm(A, B, C, M, N, K)
     seen = check(rd)
-    assert seen == dict(decided=parts(M, N), fixed=seen["fixed"], left=0, lost=0), seen
+    assert seen == dict(decided=parts(M, N), fixed=seen["fixed"], left=0, lost=0, early=0), seen
     assert_product(orc, a, b, C)
 
 
@@ -227,3 +227,34 @@ def test_small_batches_stay_on_dpx(rd, orc, count, n, tried):
     for i, C in enumerate(outs):
         got = C.cpu().numpy()
         assert np.array_equal(got[:, :n].astype(np.int32), want[i % 3]) and (got[:, n:] == -7).all()
+
+
+# both tile widths: 256 columns (the first four, two of them with several tiles per pair of CTAs) and 512; N cuts a
+# 16-byte chunk of B
+WIDTHS = [(1000, 1001, 2600), (1500, 1300, 1200), (40000, 250, 600), (39212, 249, 2600), (2100, 2301, 2130),
+          (4000, 4001, 2600)]
+
+
+@pytest.mark.parametrize("M,N,K", WIDTHS)
+def test_every_part_is_decided_on_the_tensor_cores(rd, orc, M, N, K):
+    a, b = draw(M, K, 33, 0.5, 51), draw(K, N, 33, 0.5, 52)
+    C = result(M, N)
+    rd.minplus_gemm(upload(a), upload(b), C, M, N, K)
+    seen = check(rd)
+    assert seen == dict(decided=parts(M, N), fixed=seen["fixed"], left=0, lost=0, early=0), seen
+    assert_product(orc, a, b, C)
+
+
+@pytest.mark.parametrize("M,N,K", [(39212, 249, 2600), (4000, 4001, 2600)])
+def test_the_early_look_turns_tiles_away(rd, orc, M, N, K):
+    """A's lower half holds large entries: its tiles are left an eighth of the way, the upper half's are decided, and the
+    tile across the middle at its end or by the look."""
+    a, b = draw(M, K, 33, 0.5, 53), draw(K, N, 33, 0.5, 54)
+    a[M // 2:] = np.where(a[M // 2:] == INF, INF, a[M // 2:] + 0x1000)
+    C = result(M, N)
+    rd.minplus_gemm(upload(a), upload(b), C, M, N, K)
+    seen, columns = check(rd), -(-N // 256)
+    tiles = (-(-M // 256) - (M // 2 + 255) // 256) * (1 if N <= 256 else -(-N // 512))  # whole rows of tiles below it
+    assert seen["early"] >= tiles and seen["lost"] == 0, (seen, tiles)
+    assert seen["decided"] >= M // 2 // 256 * 2 * columns and seen["decided"] + seen["left"] == parts(M, N), seen
+    assert_product(orc, a, b, C)
