@@ -938,7 +938,7 @@ static bool slices_full(int S, int64_t K) {  // every one of S K slices is non-e
 // SM, with one SM less where S is not a power of two (measured: 64 clusters of 7 do not fit in one wave).
 // The constants fit GB300's times of 12 sizes from 97 x 130 x 161 to 6000 x 5000 x 700 to 15 %.  Against the former
 // rule (wide tile, S the smallest power of two that fills a wave, slices of 256 terms and more): 97 x 130 x 161 37 ->
-// 12 us, 512^3 45 -> 17, 300 x 400 x 3000 70 -> 43, 2507 x 3001 x 1999 614 -> 520, 4096^3 2195 -> 1950; 1024^3 stays.
+// 10 us, 512^3 45 -> 17, 300 x 400 x 3000 70 -> 43, 2507 x 3001 x 1999 614 -> 520, 4096^3 2195 -> 1950; 1024^3 stays.
 GemmShape gemm_shape(int64_t M, int64_t N, int64_t K) {
   const int64_t sms = sm_count(), gpcs = 8;
   GemmShape best{1, 0, 0};
@@ -1143,7 +1143,7 @@ extern "C" rd_status rd_minplus_gemm_streamk(const int16_t* A, int64_t lda, cons
   SkLayout L;
   if (!sk_layout(M, N, K, &L)) return RD_ERR_CUDA;
   const int64_t units = L.tiles * ((K + BK - 1) / BK);
-  if (units * L.grid >= ((int64_t)1 << 32))  // many waves of whole tiles: the one-CTA-per-tile kernel
+  if (units * L.grid >= ((int64_t)1 << 32))  // many waves of whole tiles: the plain product
     return rd_minplus_gemm(A, lda, B, ldb, C, ldc, M, N, K, min_out, s);
   if (!work || (reinterpret_cast<uintptr_t>(work) & 255u) != 0) return RD_ERR_ARG;
   if (work_bytes < L.cnt_bytes + L.part_bytes) return RD_ERR_NOMEM;
