@@ -467,13 +467,16 @@ rd_status compute_cached(int m, Cached* out) {
   size_t free_b = 0, total_b = 0, least = 0;
   cudaMemGetInfo(&free_b, &total_b);
   rd_power_work_bytes(N, ld, kGammaKmax, 3, &least);
-  if (in_ring && least > total_b) {  // no form fits this device (m >= 12)
-    if (e == cudaSuccess) e = cudaErrorMemoryAllocation;
-  } else if (in_ring) {  // the plan first: it tells the size of the intermediate
+  auto make_plan = [&]() {
     size_t pbytes = 0;
-    rc = rd_split_plan_bytes(m, split_j, &pbytes);
+    if (rc == RD_OK) rc = rd_split_plan_bytes(m, split_j, &pbytes);
     if (rc == RD_OK && e == cudaSuccess) e = cudaMalloc(&plan, pbytes);
     if (rc == RD_OK && e == cudaSuccess) rc = rd_split_plan(m, split_j, plan, pbytes, &info, s);
+  };
+  if (in_ring && least > total_b) {  // no form fits this device (m >= 12)
+    if (e == cudaSuccess) e = cudaErrorMemoryAllocation;
+  } else if (in_ring && N > 8192) {  // the plan first: it tells the size of the intermediate
+    make_plan();
   }
   int slots = in_ring ? 6 : (N <= 8192) ? 16 : 8;
   size_t wbytes = 0;
@@ -506,6 +509,7 @@ rd_status compute_cached(int m, Cached* out) {
     A = reinterpret_cast<int16_t*>(static_cast<char*>(work) + off0);
   }
   if (rc == RD_OK) rc = rd_build_transfer(m, A, ld, s);
+  if (rc == RD_OK && in_ring && N <= 8192) make_plan();  // after A(G), whose kernel it overlaps
   if (rc == RD_OK && N <= kSmallN) {
     // small matrices: the whole search in one CTA
     rc = rd_power_until_periodic(A, N, ld, kGammaKmax, work, wbytes, g.data(), &k, &p, &q, s);
@@ -519,7 +523,7 @@ rd_status compute_cached(int m, Cached* out) {
     // the row-split step: A(G) (x) P_k from the row rules, in two passes
     int16_t* X = nullptr;
     const int64_t ldx = lowmem ? info.chunk_cols : ld;
-    if (rc == RD_OK) e = cudaMalloc(&X, (size_t)info.x_rows * (size_t)ldx * 2);
+    if (rc == RD_OK && e == cudaSuccess) e = cudaMalloc(&X, (size_t)info.x_rows * (size_t)ldx * 2);
     if (rc == RD_OK && e != cudaSuccess) {
       set_cuda_error(e);
       rc = (e == cudaErrorMemoryAllocation) ? RD_ERR_NOMEM : RD_ERR_CUDA;
