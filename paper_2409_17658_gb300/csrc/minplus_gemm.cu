@@ -406,6 +406,7 @@ __global__ void __launch_bounds__(NT, BNT == BN ? 2 : 3) minplus_gemm_splitk_ker
       r = make_uint4(__vmins2(r.x, t.x), __vmins2(r.y, t.y), __vmins2(r.z, t.z), __vmins2(r.w, t.w));
     }
     // the tile's word w covers columns 2w, 2w + 1: vector c8 = part * 16 + tx holds part * 128 + tx * 8 ..
+    // (what store_vec does; with it in this place the wide form spills: 1000^3 51.5 -> 55.6 us, 1500^3 129 -> 135)
     const int part = c8 / 16, tx = c8 % 16;
     const int64_t gi = m0 + row, gj = n0 + part * 128 + tx * 8;
     if (gi >= p.M || gj >= p.N) continue;
